@@ -9,103 +9,142 @@
 // read in place from the two tensors (never materialised); the 2:1 max-pool is taken in
 // the producing conv's epilogue.
 //
-// Each CTA computes a tile of TP positions x all C_out channels of one event; each
-// thread owns an 8 x 8 register block (8 consecutive positions x 8 channels). Inputs
-// are staged through shared memory in chunks of 16 channels (transposed to
-// [channel][position] so a thread's 12 halo'd inputs are three aligned float4 loads);
-// the weights of the chunk sit next to them as [tap][channel][C_out]. The sum over
-// (channel chunk, channel, tap) runs in a fixed order: results are deterministic.
+// Each CTA computes a tile of TP positions x all C_out channels of NS sequences (an event
+// is one sequence; the per-interval layout's 40 short sequences go NS = 4 or 8 to a CTA,
+// so that a CTA keeps 128 threads); each thread owns an 8 x 8 register block (8
+// consecutive positions x 8 channels; the ConvT 8 x 16). Inputs are staged through shared
+// memory in chunks of KC channels, transposed to [channel][position] so a thread's 12
+// halo'd inputs are three aligned float4 loads; the weights of the chunk sit next to them
+// as [tap][channel][C_out]. The sum over (channel, tap) runs in a fixed order: results are
+// deterministic.
+//
+// What bounds them is the FMA pipe (128 lanes per SM), if two other limits are kept off:
+//   * issue slots: the FMAs are packed two-lane instructions (each lane an fmaf), on pairs
+//     of neighbouring channels, which halves them;
+//   * the shared-memory data path, where every 16-byte load costs a warp four cycles and
+//     the 8-lane groups must hit distinct banks: a thread's 8 channels are 4 cg .. 4 cg + 3
+//     and C_out / 2 + 4 cg .. + 3, so that neighbouring lanes read neighbouring 16 bytes.
+//     (With 8 consecutive channels per thread the lanes lay 32 bytes apart: a two-way
+//     conflict that held dec3 at 74% of the shared-memory path and 0.67 of the FMA peak.)
+// The chunks are double buffered with cp.async (4-byte copies do the transposition), one
+// block barrier per chunk.
 #include "pvf_internal.cuh"
 
 namespace pvf {
 namespace {
 
-constexpr int kKC = 16;   // input channels per shared-memory chunk
+__device__ __forceinline__ uint32_t s2u(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// KC input channels per shared-memory chunk (8 where 16 would exceed the 48 KB of static
-// shared memory: the wide variant's 128- and 256-channel layers).
-template <int CA, int CB, int COUT, int TP, bool POOL, int KC = kKC>
-__global__ void __launch_bounds__((TP / 8) * (COUT / 8))
+// 4 bytes global -> shared, asynchronous; zero-filled (nothing read) when !ok
+__device__ __forceinline__ void cp4(float *dst, const float *src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s2u(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s2u(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Pitch (floats) of a staged channel row of n positions: a multiple of 4 (float4 loads) that
+// is 4 modulo 32, so that 8 channels x 4 positions written by a warp's copies hit 32 banks.
+constexpr int row_pitch(int n) { return (n + 27) / 32 * 32 + 4; }
+
+// Channel of column j (0..7) of column group cg: two runs of four, half of COUT apart.
+template <int COUT> __device__ __forceinline__ int col_of(int cg, int j) {
+    return (j < 4 ? 0 : COUT / 2) + 4 * cg + (j & 3);
+}
+
+template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC>
+__global__ void __launch_bounds__((TP / 8) * (COUT / 8) * NS, 512 / ((TP / 8) * (COUT / 8) * NS))
 k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
             const float *__restrict__ W, const float *__restrict__ bias,
             float *__restrict__ out, float *__restrict__ outp, int L) {
     constexpr int CIN = CA + CB;
-    constexpr int NCG = COUT / 8, NPG = TP / 8, NT = NCG * NPG;
-    constexpr int XR = TP + 4;              // halo'd rows of the tile
-    constexpr int XP = TP + 8;              // shared pitch (multiple of 4 floats)
+    constexpr int NCG = COUT / 8, NPG = TP / 8, NT = NCG * NPG * NS;
+    constexpr int XR = TP + 4;              // halo'd rows of a sequence's tile
+    constexpr int XP = row_pitch(NS * XR);
     static_assert(CA % KC == 0 && CB % KC == 0 && KC % 4 == 0, "channel chunks must not straddle");
-    constexpr int Q = KC / 4;               // float4 per halo'd row of a chunk
-    __shared__ __align__(16) float xs[KC][XP];
-    __shared__ __align__(16) float ws[5][KC][COUT];
+    static_assert(COUT % 16 == 0 && TP % 8 == 0, "tiles");
+    __shared__ __align__(16) float xs[2][KC][XP];
+    __shared__ __align__(16) float ws[2][5][KC][COUT];
 
     const int tid = threadIdx.x;
-    const int cg = tid % NCG, pg = tid / NCG;
-    const int e = blockIdx.y;
+    const int cg = tid % NCG, pg = tid / NCG % NPG, sq = tid / (NCG * NPG);
+    const int64_t e0 = (int64_t)blockIdx.y * NS;      // first sequence of this CTA
     const int p0 = blockIdx.x * TP;
     const int64_t rowsE = padded_rows(L);
 
-    float acc[8][8];
-#pragma unroll
-    for (int qi = 0; qi < 8; ++qi) {
-        const float b = bias[cg * 8 + qi];
-#pragma unroll
-        for (int pi = 0; pi < 8; ++pi) acc[pi][qi] = b;
-    }
-
-    for (int kc = 0; kc < CIN; kc += KC) {
+    auto stage = [&](int kc, int buf) {
         const bool fromA = kc < CA;
         const int C = fromA ? CA : CB;
-        const int coff = fromA ? kc : kc - CA;
-        const float *src = (fromA ? inA : inB) + (size_t)e * rowsE * C + coff;
-        // tile row r <-> event row p0 - 2 + r <-> storage row p0 + r
-        for (int idx = tid; idx < XR * Q; idx += NT) {
-            const int r = idx / Q, c4 = idx % Q;
+        const float *src = (fromA ? inA : inB) + (fromA ? kc : kc - CA);
+        // tile row r of sequence s <-> position p0 - 2 + r <-> storage row p0 + r
+        for (int idx = tid; idx < NS * XR * KC; idx += NT) {
+            const int k = idx % KC, rr = idx / KC;
+            const int s = NS == 1 ? 0 : rr / XR, r = NS == 1 ? rr : rr % XR;
             const int64_t srow = (int64_t)p0 + r;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (srow < rowsE) v = *reinterpret_cast<const float4 *>(src + srow * C + 4 * c4);
-            xs[4 * c4 + 0][r] = v.x;
-            xs[4 * c4 + 1][r] = v.y;
-            xs[4 * c4 + 2][r] = v.z;
-            xs[4 * c4 + 3][r] = v.w;
+            const bool ok = srow < rowsE;
+            cp4(&xs[buf][k][rr], src + ((e0 + s) * rowsE + (ok ? srow : 0)) * C + k, ok);
         }
         for (int idx = tid; idx < 5 * KC * COUT / 4; idx += NT) {
             const int t = idx / (KC * COUT / 4), rem = idx % (KC * COUT / 4);
-            const int k = rem / (COUT / 4), c4 = rem % (COUT / 4);
-            reinterpret_cast<float4 *>(&ws[t][k][0])[c4] =
-                reinterpret_cast<const float4 *>(W + ((size_t)t * CIN + kc + k) * COUT)[c4];
+            cp16(reinterpret_cast<float4 *>(&ws[buf][t][0][0]) + rem,
+                 reinterpret_cast<const float4 *>(W + ((size_t)t * CIN + kc) * COUT) + rem);
         }
-        __syncthreads();
-#pragma unroll 2
+    };
+
+    stage(0, 0);
+    float2 acc[8][4];                        // [position][channel pair]
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 b = make_float2(bias[col_of<COUT>(cg, 2 * q)], bias[col_of<COUT>(cg, 2 * q + 1)]);
+#pragma unroll
+        for (int pi = 0; pi < 8; ++pi) acc[pi][q] = b;
+    }
+
+    constexpr int NCH = CIN / KC;
+#pragma unroll 1
+    for (int c = 0; c < NCH; ++c) {
+        const int buf = c & 1;
+        cp_wait_all();
+        __syncthreads();                     // chunk c staged; the other buffer is no longer read
+        if (c + 1 < NCH) stage((c + 1) * KC, buf ^ 1);
+#pragma unroll 1
         for (int k = 0; k < KC; ++k) {
             float xv[12];
-            const float4 *xr = reinterpret_cast<const float4 *>(&xs[k][pg * 8]);
+            const float4 *xr = reinterpret_cast<const float4 *>(&xs[buf][k][sq * XR + pg * 8]);
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                float4 v = xr[i];
+                const float4 v = xr[i];
                 xv[4 * i] = v.x; xv[4 * i + 1] = v.y; xv[4 * i + 2] = v.z; xv[4 * i + 3] = v.w;
             }
 #pragma unroll
             for (int t = 0; t < 5; ++t) {
-                const float4 *wr = reinterpret_cast<const float4 *>(&ws[t][k][cg * 8]);
-                const float4 wa = wr[0], wb = wr[1];
-                const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                const float4 wa = *reinterpret_cast<const float4 *>(&ws[buf][t][k][4 * cg]);
+                const float4 wb = *reinterpret_cast<const float4 *>(&ws[buf][t][k][COUT / 2 + 4 * cg]);
+                const float2 wv[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
+                                      make_float2(wb.z, wb.w)};
 #pragma unroll
-                for (int pi = 0; pi < 8; ++pi)
+                for (int pi = 0; pi < 8; ++pi) {
+                    const float2 x2 = make_float2(xv[pi + t], xv[pi + t]);
 #pragma unroll
-                    for (int qi = 0; qi < 8; ++qi) acc[pi][qi] = fmaf(xv[pi + t], wv[qi], acc[pi][qi]);
+                    for (int q = 0; q < 4; ++q) acc[pi][q] = __ffma2_rn(x2, wv[q], acc[pi][q]);
+                }
             }
         }
-        __syncthreads();
     }
 
+    const int64_t e = e0 + sq;
     float *ob = out + (size_t)e * rowsE * COUT;
 #pragma unroll
     for (int pi = 0; pi < 8; ++pi) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[pi][q] = make_float2(leaky(acc[pi][q].x), leaky(acc[pi][q].y));
         const int p = p0 + pg * 8 + pi;
         if (p < L) {
-            float4 *d = reinterpret_cast<float4 *>(ob + (size_t)(p + kPad) * COUT + cg * 8);
-            d[0] = make_float4(leaky(acc[pi][0]), leaky(acc[pi][1]), leaky(acc[pi][2]), leaky(acc[pi][3]));
-            d[1] = make_float4(leaky(acc[pi][4]), leaky(acc[pi][5]), leaky(acc[pi][6]), leaky(acc[pi][7]));
+            float *d = ob + (size_t)(p + kPad) * COUT + 4 * cg;
+            *reinterpret_cast<float4 *>(d) = make_float4(acc[pi][0].x, acc[pi][0].y, acc[pi][1].x, acc[pi][1].y);
+            *reinterpret_cast<float4 *>(d + COUT / 2) =
+                make_float4(acc[pi][2].x, acc[pi][2].y, acc[pi][3].x, acc[pi][3].y);
         }
     }
     if constexpr (POOL) {
@@ -115,102 +154,123 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
         for (int pi = 0; pi < 8; pi += 2) {
             const int p = p0 + pg * 8 + pi;
             if (p + 1 < L) {
-                float v[8];
+                float2 v[4];
 #pragma unroll
-                for (int qi = 0; qi < 8; ++qi) v[qi] = fmaxf(leaky(acc[pi][qi]), leaky(acc[pi + 1][qi]));
-                float4 *d = reinterpret_cast<float4 *>(pb + (size_t)(p / 2 + kPad) * COUT + cg * 8);
-                d[0] = make_float4(v[0], v[1], v[2], v[3]);
-                d[1] = make_float4(v[4], v[5], v[6], v[7]);
+                for (int q = 0; q < 4; ++q)
+                    v[q] = make_float2(fmaxf(acc[pi][q].x, acc[pi + 1][q].x), fmaxf(acc[pi][q].y, acc[pi + 1][q].y));
+                float *d = pb + (size_t)(p / 2 + kPad) * COUT + 4 * cg;
+                *reinterpret_cast<float4 *>(d) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+                *reinterpret_cast<float4 *>(d + COUT / 2) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
             }
         }
     }
-    // pad rows of this event: written by the first and the last tile
+    // pad rows of each sequence: written by its first and its last tile
     // (a single tile is both: it writes both sides)
     const bool first = blockIdx.x == 0, last = blockIdx.x == gridDim.x - 1;
 #pragma unroll 1
     for (int side = 0; side < 2; ++side) {
         if (!(side == 0 ? first : last)) continue;
         const int base = side == 0 ? 0 : L + kPad;
-        for (int i = tid; i < 2 * COUT; i += NT) ob[(size_t)base * COUT + i] = 0.0f;
-        if constexpr (POOL) {
-            const int Lp = L / 2;
-            float *pb = outp + (size_t)e * padded_rows(Lp) * COUT;
-            const int pbase = side == 0 ? 0 : Lp + kPad;
-            for (int i = tid; i < 2 * COUT; i += NT) pb[(size_t)pbase * COUT + i] = 0.0f;
+        for (int i = tid; i < NS * 2 * COUT; i += NT) {
+            const int64_t es = e0 + i / (2 * COUT);
+            out[((size_t)es * rowsE + base) * COUT + i % (2 * COUT)] = 0.0f;
+            if constexpr (POOL) {
+                const int Lp = L / 2;
+                const int pbase = side == 0 ? 0 : Lp + kPad;
+                outp[((size_t)es * padded_rows(Lp) + pbase) * COUT + i % (2 * COUT)] = 0.0f;
+            }
         }
     }
 }
 
 // ConvTranspose1d k2 s2 + LeakyReLU: out[2i + r][co] = lrelu(b[co] + sum_ci W[ci][r][co] in[i][ci]).
-// A GEMM per event with M = input positions, N = 2 * C_out (column n = r * C_out + co).
-template <int CIN, int COUT, int TP>
-__global__ void __launch_bounds__((TP / 8) * (2 * COUT / 8))
+// A GEMM per event with M = input positions, N = 2 * C_out (column n = r * C_out + co). A
+// thread owns 8 positions x 16 columns (four runs of four, N / 4 apart): per channel six
+// 16-byte shared loads for 64 packed FMAs (8 x 8 blocks would need as many load cycles as
+// FMA cycles).
+template <int CIN, int COUT, int TP, int NS, int KC>
+__global__ void __launch_bounds__((TP / 8) * (2 * COUT / 16) * NS, 256 / ((TP / 8) * (2 * COUT / 16) * NS))
 k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
             const float *__restrict__ bias, float *__restrict__ out, int Lin) {
     constexpr int N = 2 * COUT;
-    constexpr int NCG = N / 8, NPG = TP / 8, NT = NCG * NPG;
-    constexpr int XP = TP + 4;
-    __shared__ __align__(16) float xs[kKC][XP];
-    __shared__ __align__(16) float ws[kKC][N];
+    constexpr int NCG = N / 16, NPG = TP / 8, NT = NCG * NPG * NS;
+    constexpr int XP = row_pitch(NS * TP);
+    static_assert(CIN % KC == 0 && KC % 8 == 0 && N % 32 == 0, "channel chunks");
+    __shared__ __align__(16) float xs[2][KC][XP];
+    __shared__ __align__(16) float ws[2][KC][N];
 
     const int tid = threadIdx.x;
-    const int cg = tid % NCG, pg = tid / NCG;
-    const int e = blockIdx.y;
+    const int cg = tid % NCG, pg = tid / NCG % NPG, sq = tid / (NCG * NPG);
+    const int64_t e0 = (int64_t)blockIdx.y * NS;
     const int p0 = blockIdx.x * TP;
     const int64_t rowsIn = padded_rows(Lin);
     const int Lout = 2 * Lin;
     const int64_t rowsOut = padded_rows(Lout);
-    const int rr = (cg * 8) / COUT;        // phase r of this thread's columns
-    const int co0 = (cg * 8) % COUT;
 
-    float acc[8][8];
+    auto stage = [&](int kc, int buf) {
+        // 8 channels at a time: 32 contiguous bytes per position, distinct banks per warp
+        for (int idx = tid; idx < NS * TP * KC; idx += NT) {
+            const int k = idx % 8 + idx / (8 * NS * TP) * 8, rr = idx / 8 % (NS * TP);
+            const int s = NS == 1 ? 0 : rr / TP, p = p0 + (NS == 1 ? rr : rr % TP);
+            const bool ok = p < Lin;
+            cp4(&xs[buf][k][rr], in + ((e0 + s) * rowsIn + (ok ? p + kPad : 0)) * CIN + kc + k, ok);
+        }
+        for (int idx = tid; idx < KC * N / 4; idx += NT)
+            cp16(reinterpret_cast<float4 *>(&ws[buf][0][0]) + idx,
+                 reinterpret_cast<const float4 *>(W + (size_t)kc * N) + idx);
+    };
+
+    stage(0, 0);
+    float2 acc[8][8];                        // [position][column pair]
 #pragma unroll
-    for (int qi = 0; qi < 8; ++qi) {
-        const float b = bias[co0 + qi];
+    for (int g = 0; g < 4; ++g) {
+        const int co = (g * (N / 4) + 4 * cg) % COUT;
 #pragma unroll
-        for (int pi = 0; pi < 8; ++pi) acc[pi][qi] = b;
+        for (int h = 0; h < 2; ++h) {
+            const float2 b = make_float2(bias[co + 2 * h], bias[co + 2 * h + 1]);
+#pragma unroll
+            for (int pi = 0; pi < 8; ++pi) acc[pi][2 * g + h] = b;
+        }
     }
-    const float *src = in + (size_t)e * rowsIn * CIN;
-    for (int kc = 0; kc < CIN; kc += kKC) {
-        for (int idx = tid; idx < TP * (kKC / 4); idx += NT) {
-            const int r = idx >> 2, c4 = idx & 3;
-            const int p = p0 + r;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p < Lin) v = *reinterpret_cast<const float4 *>(src + (size_t)(p + kPad) * CIN + kc + 4 * c4);
-            xs[4 * c4 + 0][r] = v.x;
-            xs[4 * c4 + 1][r] = v.y;
-            xs[4 * c4 + 2][r] = v.z;
-            xs[4 * c4 + 3][r] = v.w;
-        }
-        for (int idx = tid; idx < kKC * N / 4; idx += NT) {
-            const int k = idx / (N / 4), c4 = idx % (N / 4);
-            reinterpret_cast<float4 *>(&ws[k][0])[c4] =
-                reinterpret_cast<const float4 *>(W + (size_t)(kc + k) * N)[c4];
-        }
+    constexpr int NCH = CIN / KC;
+#pragma unroll 1
+    for (int c = 0; c < NCH; ++c) {
+        const int buf = c & 1;
+        cp_wait_all();
         __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < kKC; ++k) {
-            const float4 *xr = reinterpret_cast<const float4 *>(&xs[k][pg * 8]);
+        if (c + 1 < NCH) stage((c + 1) * KC, buf ^ 1);
+#pragma unroll 2
+        for (int k = 0; k < KC; ++k) {
+            const float4 *xr = reinterpret_cast<const float4 *>(&xs[buf][k][sq * TP + pg * 8]);
             const float4 xa = xr[0], xb = xr[1];
             const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-            const float4 *wr = reinterpret_cast<const float4 *>(&ws[k][cg * 8]);
-            const float4 wa = wr[0], wb = wr[1];
-            const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+            float2 wv[8];
 #pragma unroll
-            for (int pi = 0; pi < 8; ++pi)
+            for (int g = 0; g < 4; ++g) {
+                const float4 w4 = *reinterpret_cast<const float4 *>(&ws[buf][k][g * (N / 4) + 4 * cg]);
+                wv[2 * g] = make_float2(w4.x, w4.y);
+                wv[2 * g + 1] = make_float2(w4.z, w4.w);
+            }
 #pragma unroll
-                for (int qi = 0; qi < 8; ++qi) acc[pi][qi] = fmaf(xv[pi], wv[qi], acc[pi][qi]);
+            for (int pi = 0; pi < 8; ++pi) {
+                const float2 x2 = make_float2(xv[pi], xv[pi]);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc[pi][q] = __ffma2_rn(x2, wv[q], acc[pi][q]);
+            }
         }
-        __syncthreads();
     }
-    float *ob = out + (size_t)e * rowsOut * COUT;
+    float *ob = out + (size_t)(e0 + sq) * rowsOut * COUT;
 #pragma unroll
     for (int pi = 0; pi < 8; ++pi) {
         const int i = p0 + pg * 8 + pi;
         if (i < Lin) {
-            float4 *d = reinterpret_cast<float4 *>(ob + (size_t)(2 * i + rr + kPad) * COUT + co0);
-            d[0] = make_float4(leaky(acc[pi][0]), leaky(acc[pi][1]), leaky(acc[pi][2]), leaky(acc[pi][3]));
-            d[1] = make_float4(leaky(acc[pi][4]), leaky(acc[pi][5]), leaky(acc[pi][6]), leaky(acc[pi][7]));
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const int n = g * (N / 4) + 4 * cg;      // column n: output row 2 i + n / COUT
+                const float2 a = acc[pi][2 * g], b = acc[pi][2 * g + 1];
+                *reinterpret_cast<float4 *>(ob + (size_t)(2 * i + n / COUT + kPad) * COUT + n % COUT) =
+                    make_float4(leaky(a.x), leaky(a.y), leaky(b.x), leaky(b.y));
+            }
         }
     }
     const bool first = blockIdx.x == 0, last = blockIdx.x == gridDim.x - 1;
@@ -218,69 +278,73 @@ k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
     for (int side = 0; side < 2; ++side) {   // a single tile is both first and last
         if (!(side == 0 ? first : last)) continue;
         const int base = side == 0 ? 0 : Lout + kPad;
-        for (int i = tid; i < 2 * COUT; i += NT) ob[(size_t)base * COUT + i] = 0.0f;
+        for (int i = tid; i < NS * 2 * COUT; i += NT)
+            out[((size_t)(e0 + i / (2 * COUT)) * rowsOut + base) * COUT + i % (2 * COUT)] = 0.0f;
     }
 }
 
-template <int CA, int CB, int COUT, int TP, bool POOL, int KC = kKC>
+// n: sequences (a multiple of NS)
+template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC>
 cudaError_t conv5(const void *a, const void *b, const float *W, const float *bias, void *out,
                   void *outp, int L, int n, cudaStream_t s) {
-    dim3 grid((L + TP - 1) / TP, n), block((TP / 8) * (COUT / 8));
-    k_conv5_f32<CA, CB, COUT, TP, POOL, KC><<<grid, block, 0, s>>>(
+    dim3 grid((L + TP - 1) / TP, n / NS), block((TP / 8) * (COUT / 8) * NS);
+    k_conv5_f32<CA, CB, COUT, TP, NS, POOL, KC><<<grid, block, 0, s>>>(
         (const float *)a, (const float *)b, W, bias, (float *)out, (float *)outp, L);
     return cudaGetLastError();
 }
 
-template <int CIN, int COUT, int TP>
+template <int CIN, int COUT, int TP, int NS, int KC>
 cudaError_t convT(const void *in, const float *W, const float *bias, void *out, int Lin, int n,
                   cudaStream_t s) {
-    dim3 grid((Lin + TP - 1) / TP, n), block((TP / 8) * (2 * COUT / 8));
-    k_convT_f32<CIN, COUT, TP><<<grid, block, 0, s>>>((const float *)in, W, bias, (float *)out, Lin);
+    dim3 grid((Lin + TP - 1) / TP, n / NS), block((TP / 8) * (2 * COUT / 16) * NS);
+    k_convT_f32<CIN, COUT, TP, NS, KC><<<grid, block, 0, s>>>((const float *)in, W, bias, (float *)out, Lin);
     return cudaGetLastError();
 }
 
 // The layer sequence for base width C (levels C, 2C, 4C, 8C). Tiles halve as the channel
-// counts double, so every CTA keeps (TP / 8) x (C_out / 8) = 128 threads; in the wide
-// variant the 2C-, 4C- and 8C-input convolutions stage 8 channels per chunk so that their
-// weights fit the 48 KB of static shared memory (enc4 at C = 32: 40 KB).
+// counts double, so every CTA keeps 128 threads. Channels per chunk: 8 (double buffered,
+// weights and inputs fit the 48 KB of static shared memory), 4 for the 256-channel output.
 template <int C>
 cudaError_t run_f32(const ConvF32Weights &w, const UnetBuffers &b, int n, cudaStream_t s,
                     const ProfHook *prof) {
-    constexpr int KW = C > kC0 ? 8 : kKC;
+    constexpr int R = kC0;                       // tile sizes are for base width R, halved at 2 R
+    constexpr int K4 = C > kC0 ? 4 : 8;
     cudaError_t err;
 #define PVF_TRY(name, x) do { ProfScope ps_(prof, name, s); err = (x); if (err != cudaSuccess) return err; } while (0)
     // each tensor is packed in its slot with its own per-event stride (L + 4) * C
-    PVF_TRY("enc2", (conv5<C, 0, 2 * C, 256 * 16 / C, true>(b.s0, nullptr, w.w[0], w.b[0], b.e2, b.s1, 2000, n, s)));
-    PVF_TRY("enc3", (conv5<2 * C, 0, 4 * C, 128 * 16 / C, true, KW>(b.s1, nullptr, w.w[1], w.b[1], b.e3, b.s0, 1000, n, s)));
-    PVF_TRY("enc4", (conv5<4 * C, 0, 8 * C, 64 * 16 / C, false, KW>(b.s0, nullptr, w.w[2], w.b[2], b.deep, nullptr, 500, n, s)));
-    PVF_TRY("up3", (convT<8 * C, 4 * C, 64 * 16 / C>(b.deep, w.uw[0], w.ub[0], b.up, 500, n, s)));
-    PVF_TRY("dec3", (conv5<4 * C, 4 * C, 4 * C, 128 * 16 / C, false, KW>(b.up, b.e3, w.w[3], w.b[3], b.deep, nullptr, 1000, n, s)));
-    PVF_TRY("up2", (convT<4 * C, 2 * C, 128 * 16 / C>(b.deep, w.uw[1], w.ub[1], b.up, 1000, n, s)));
-    PVF_TRY("dec2", (conv5<2 * C, 2 * C, 2 * C, 256 * 16 / C, false>(b.up, b.e2, w.w[4], w.b[4], b.deep, nullptr, 2000, n, s)));
-    PVF_TRY("up1", (convT<2 * C, C, 256 * 16 / C>(b.deep, w.uw[2], w.ub[2], b.up, 2000, n, s)));
-    PVF_TRY("dec1", (conv5<C, C, C, 512 * 16 / C, false>(b.up, b.e1, w.w[5], w.b[5], b.deep, nullptr, 4000, n, s)));
+    PVF_TRY("enc2", (conv5<C, 0, 2 * C, 256 * R / C, 1, true, 8>(b.s0, nullptr, w.w[0], w.b[0], b.e2, b.s1, 2000, n, s)));
+    PVF_TRY("enc3", (conv5<2 * C, 0, 4 * C, 128 * R / C, 1, true, 8>(b.s1, nullptr, w.w[1], w.b[1], b.e3, b.s0, 1000, n, s)));
+    PVF_TRY("enc4", (conv5<4 * C, 0, 8 * C, 64 * R / C, 1, false, K4>(b.s0, nullptr, w.w[2], w.b[2], b.deep, nullptr, 500, n, s)));
+    PVF_TRY("up3", (convT<8 * C, 4 * C, 128 * R / C, 1, 16>(b.deep, w.uw[0], w.ub[0], b.up, 500, n, s)));
+    PVF_TRY("dec3", (conv5<4 * C, 4 * C, 4 * C, 128 * R / C, 1, false, 8>(b.up, b.e3, w.w[3], w.b[3], b.deep, nullptr, 1000, n, s)));
+    PVF_TRY("up2", (convT<4 * C, 2 * C, 256 * R / C, 1, 16>(b.deep, w.uw[1], w.ub[1], b.up, 1000, n, s)));
+    PVF_TRY("dec2", (conv5<2 * C, 2 * C, 2 * C, 256 * R / C, 1, false, 8>(b.up, b.e2, w.w[4], w.b[4], b.deep, nullptr, 2000, n, s)));
+    PVF_TRY("up1", (convT<2 * C, C, 512 * R / C, 1, 8>(b.deep, w.uw[2], w.ub[2], b.up, 2000, n, s)));
+    PVF_TRY("dec1", (conv5<C, C, C, 512 * R / C, 1, false, 8>(b.up, b.e1, w.w[5], w.b[5], b.deep, nullptr, 4000, n, s)));
 #undef PVF_TRY
     return cudaSuccess;
 }
 
 // The per-interval layout: kSlices sequences of kIvLen bins per event (104, 52, 26, 13
-// positions per level), each layer one small tile per sequence (32 threads per CTA).
+// positions per level), each layer one small tile per sequence, 4 or 8 sequences per CTA
+// (kSlices is a multiple of both, so every group is full).
 template <int C>
 cudaError_t run_f32_iv(const ConvF32Weights &w, const UnetBuffers &b, int n, cudaStream_t s,
                        const ProfHook *prof) {
     constexpr int L1 = kIvLen, L2 = L1 / 2, L3 = L1 / 4, L4 = L1 / 8;
+    static_assert(kSlices % 8 == 0, "full groups of sequences");
     const int ns = n * kSlices;                  // at most 64000 (the plan caps the chunk)
     cudaError_t err;
 #define PVF_TRY(name, x) do { ProfScope ps_(prof, name, s); err = (x); if (err != cudaSuccess) return err; } while (0)
-    PVF_TRY("enc2", (conv5<C, 0, 2 * C, 64, true>(b.s0, nullptr, w.w[0], w.b[0], b.e2, b.s1, L2, ns, s)));
-    PVF_TRY("enc3", (conv5<2 * C, 0, 4 * C, 32, true>(b.s1, nullptr, w.w[1], w.b[1], b.e3, b.s0, L3, ns, s)));
-    PVF_TRY("enc4", (conv5<4 * C, 0, 8 * C, 16, false>(b.s0, nullptr, w.w[2], w.b[2], b.deep, nullptr, L4, ns, s)));
-    PVF_TRY("up3", (convT<8 * C, 4 * C, 16>(b.deep, w.uw[0], w.ub[0], b.up, L4, ns, s)));
-    PVF_TRY("dec3", (conv5<4 * C, 4 * C, 4 * C, 32, false>(b.up, b.e3, w.w[3], w.b[3], b.deep, nullptr, L3, ns, s)));
-    PVF_TRY("up2", (convT<4 * C, 2 * C, 32>(b.deep, w.uw[1], w.ub[1], b.up, L3, ns, s)));
-    PVF_TRY("dec2", (conv5<2 * C, 2 * C, 2 * C, 64, false>(b.up, b.e2, w.w[4], w.b[4], b.deep, nullptr, L2, ns, s)));
-    PVF_TRY("up1", (convT<2 * C, C, 64>(b.deep, w.uw[2], w.ub[2], b.up, L2, ns, s)));
-    PVF_TRY("dec1", (conv5<C, C, C, 128, false>(b.up, b.e1, w.w[5], w.b[5], b.deep, nullptr, L1, ns, s)));
+    PVF_TRY("enc2", (conv5<C, 0, 2 * C, 64, 4, true, 8>(b.s0, nullptr, w.w[0], w.b[0], b.e2, b.s1, L2, ns, s)));
+    PVF_TRY("enc3", (conv5<2 * C, 0, 4 * C, 32, 4, true, 8>(b.s1, nullptr, w.w[1], w.b[1], b.e3, b.s0, L3, ns, s)));
+    PVF_TRY("enc4", (conv5<4 * C, 0, 8 * C, 16, 4, false, 8>(b.s0, nullptr, w.w[2], w.b[2], b.deep, nullptr, L4, ns, s)));
+    PVF_TRY("up3", (convT<8 * C, 4 * C, 16, 8, 16>(b.deep, w.uw[0], w.ub[0], b.up, L4, ns, s)));
+    PVF_TRY("dec3", (conv5<4 * C, 4 * C, 4 * C, 32, 4, false, 8>(b.up, b.e3, w.w[3], w.b[3], b.deep, nullptr, L3, ns, s)));
+    PVF_TRY("up2", (convT<4 * C, 2 * C, 32, 8, 16>(b.deep, w.uw[1], w.ub[1], b.up, L3, ns, s)));
+    PVF_TRY("dec2", (conv5<2 * C, 2 * C, 2 * C, 64, 4, false, 8>(b.up, b.e2, w.w[4], w.b[4], b.deep, nullptr, L2, ns, s)));
+    PVF_TRY("up1", (convT<2 * C, C, 64, 8, 8>(b.deep, w.uw[2], w.ub[2], b.up, L2, ns, s)));
+    PVF_TRY("dec1", (conv5<C, C, C, 128, 4, false, 8>(b.up, b.e1, w.w[5], w.b[5], b.deep, nullptr, L1, ns, s)));
 #undef PVF_TRY
     return cudaSuccess;
 }
