@@ -242,7 +242,7 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
                 hv[k] = (p >= 0 && p < kBins) ? shist[p] : 0.0f;
             }
         }
-        float v0[8], v1[8], vp[8];
+        float v0[8], v1[8];
         // channel pairs (j, j + 1) as one packed two-lane FMA (each lane an fmaf, in the
         // same tap order): half the FMA instructions, identical results
 #pragma unroll
@@ -254,17 +254,32 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
                 a0 = __ffma2_rn(wt, make_float2(hv[t], hv[t]), a0);
                 a1 = __ffma2_rn(wt, make_float2(hv[t + 1], hv[t + 1]), a1);
             }
-            v0[j] = leaky(a0.x); v0[j + 1] = leaky(a0.y);
-            v1[j] = leaky(a1.x); v1[j + 1] = leaky(a1.y);
+            a0 = leaky2(a0);
+            a1 = leaky2(a1);
+            v0[j] = a0.x; v0[j + 1] = a0.y;
+            v1[j] = a1.x; v1[j + 1] = a1.y;
         }
+        if constexpr (AMAX) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            vp[j] = fmaxf(v0[j], v1[j]);
-            if constexpr (AMAX) vmax = fmaxf(vmax, fmaxf(fabsf(v0[j]), fabsf(v1[j])));
+            for (int j = 0; j < 8; ++j) vmax = fmaxf(vmax, fmaxf(fabsf(v0[j]), fabsf(v1[j])));
         }
-        store_half8<T>(a.e1, e, rows1, r1, h, v0, inv);
-        store_half8<T>(a.e1, e, rows1, r1 + 1, h, v1, inv);
-        store_half8<T>(a.p1, e, rows2, r2, h, vp, inv);
+        if constexpr (sizeof(T) == 2) {
+            // the pooled row from the packed rows: the maximum of the rounded values is the
+            // rounded maximum
+            const uint4 r0 = pack8<T>(v0), r1v = pack8<T>(v1);
+            unsigned char *d1 = reinterpret_cast<unsigned char *>(a.e1) + planar_off(e, h, 2, rows1, r1);
+            *reinterpret_cast<uint4 *>(d1) = r0;
+            *reinterpret_cast<uint4 *>(d1 + 16) = r1v;
+            *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.p1) + planar_off(e, h, 2, rows2, r2)) =
+                make_uint4(max2<T>(r0.x, r1v.x), max2<T>(r0.y, r1v.y), max2<T>(r0.z, r1v.z), max2<T>(r0.w, r1v.w));
+        } else {
+            float vp[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) vp[j] = fmaxf(v0[j], v1[j]);
+            store_half8<T>(a.e1, e, rows1, r1, h, v0, inv);
+            store_half8<T>(a.e1, e, rows1, r1 + 1, h, v1, inv);
+            store_half8<T>(a.p1, e, rows2, r2, h, vp, inv);
+        }
     }
     if constexpr (AMAX) {   // calibration: integer max on the float bits (order-independent)
 #pragma unroll

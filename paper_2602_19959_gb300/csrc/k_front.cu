@@ -175,8 +175,12 @@ __global__ void __launch_bounds__(kThreads) k_front(FrontArgs a) {
             for (int i = tid; i < kBins / 4; i += kThreads) dst[i] = src[i];
         }
 
-        if constexpr (ENC1 && IV) enc1_pool_windows_f32<kThreads, C0>(a, e, tid, shist, senc);
-        else if constexpr (ENC1) enc1_pool<T, kThreads, false, C0>(a, e, tid, shist, senc);
+        if constexpr (ENC1) {
+            if (a.e1) {      // null: the histogram alone was asked for
+                if constexpr (IV) enc1_pool_windows_f32<kThreads, C0>(a, e, tid, shist, senc);
+                else enc1_pool<T, kThreads, false, C0>(a, e, tid, shist, senc);
+            }
+        }
         __syncthreads();                   // shist and the sort arrays are reused next event
     }
 }

@@ -218,9 +218,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
                             float v[32];
                             tmem_ld16(dcol, *reinterpret_cast<float(*)[16]>(v));
                             tmem_ld16(dcol + 16, *reinterpret_cast<float(*)[16]>(v + 16));
-                            const float *b = sbias + l * kFcHidden;
+                            float b[32];
+                            const float4 *b4 = reinterpret_cast<const float4 *>(sbias + l * kFcHidden);
 #pragma unroll
-                            for (int o = 0; o < kFcHidden; ++o) v[o] = leaky(v[o] + b[o]);
+                            for (int o = 0; o < kFcHidden / 4; ++o) {
+                                const float4 x = b4[o];
+                                b[4 * o] = x.x; b[4 * o + 1] = x.y; b[4 * o + 2] = x.z; b[4 * o + 3] = x.w;
+                            }
+                            bias_leaky(v, b);
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
                                 *reinterpret_cast<uint4 *>(hrow + k * kPlane) = pack8<FT>(v + 8 * k);
@@ -301,7 +306,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
             const float4 *src = reinterpret_cast<const float4 *>(shist);
             for (int i = tid; i < kBins / 4; i += kT) dst[i] = src[i];
         }
-        if (a.iv) enc1_pool<T, kT, true, kC0, true>(a, e, tid, shist, senc);
+        if (!a.e1) {}                                    // the histogram alone was asked for
+        else if (a.iv) enc1_pool<T, kT, true, kC0, true>(a, e, tid, shist, senc);
         else if (a.c0 == kC0Max) enc1_pool<T, kT, false, kC0Max>(a, e, tid, shist, senc);   // the wide network
         else enc1_pool<T, kT>(a, e, tid, shist, senc);
         if (tid == 0) {

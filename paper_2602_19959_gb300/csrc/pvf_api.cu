@@ -523,8 +523,8 @@ static cudaError_t run_chunk(pvf_handle *h, const pvf_tracks_soa *tracks, const 
         a.enc1 = h->enc1;
         a.hist_in = hist_in;
         a.hist_out = hist_out;
-        a.e1 = h->buf.e1;
-        a.p1 = h->buf.s0;
+        a.e1 = run_unet ? h->buf.e1 : nullptr;      // without the UNet nobody reads e1 and p1
+        a.p1 = run_unet ? h->buf.s0 : nullptr;
         a.e1_inv_scale = 1.0f / h->act_scale[kScaleL1];
         a.ev_flag = flags;
         a.status = status;
