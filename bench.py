@@ -78,8 +78,9 @@ def kernel_table(form, c0=16, iv=False):
     t = {}
     e1 = q * (c1 * (L0 + 4) + c1 * (L1 + 4))            # e1 and p1 written by the front kernel
     t["front"] = (0, q * L0 * c1 * 5, e1 * es)          # enc1 on CUDA cores; + the FC, + 36 B per track
-    m, r, w = scaled(conv_io(L1, c1, c2, pool=True)); t["enc2"] = entry(m, (r + w) * es)
-    m, r, w = scaled(conv_io(L2, c2, c3, pool=True)); t["enc3"] = entry(m, (r + w) * es)
+    if form == "fp32" or c0 == 32 or iv:
+        m, r, w = scaled(conv_io(L1, c1, c2, pool=True)); t["enc2"] = entry(m, (r + w) * es)
+        m, r, w = scaled(conv_io(L2, c2, c3, pool=True)); t["enc3"] = entry(m, (r + w) * es)
     if form == "fp32":
         m, r, w = scaled(conv_io(L3, c3, c4)); t["enc4"] = entry(m, (r + w) * es)
         m, r, w = scaled(convT_io(L3, c4, c3)); t["up3"] = entry(m, (r + w) * es)
@@ -103,7 +104,11 @@ def kernel_table(form, c0=16, iv=False):
         t["tail"] = (0, 0, 16000)
     else:
         m1, r1, _ = scaled(conv_io(L3, c3, c4)); m2, _, w2 = scaled(convT_io(L3, c4, c3))
-        t["enc4_up3"] = entry(m1 + m2, (r1 + w2) * es)
+        if iv:
+            t["enc4_up3"] = entry(m1 + m2, (r1 + w2) * es)
+        else:   # one kernel from p1 to e2, e3 and u3: p2 and p3 stay in shared memory
+            m3, r3, w3 = conv_io(L1, c1, c2); m4, _, w4 = conv_io(L2, c2, c3)
+            t["enc_up3"] = entry(m1 + m2 + m3 + m4, (r3 + w3 + w4 + w2) * es)
         m1, r1, _ = scaled(conv_io(L2, 2 * c3, c3)); m2, _, w2 = scaled(convT_io(L2, c3, c2))
         t["dec3_up2"] = entry(m1 + m2, (r1 + w2) * es)
         m1, r1, _ = scaled(conv_io(L1, 2 * c2, c2)); m2, _, w2 = scaled(convT_io(L1, c2, c1))

@@ -85,7 +85,9 @@ typedef struct {
                                       launches of at most 4 events per SM, else 4. The
                                       float32 front: 1..2                                   */
     int32_t conv_ctas_per_sm[6];   /* tensor-core forms: enc2, enc3, enc4_up3, dec3_up2,
-                                      dec2_up1, dec1_final                                    */
+                                      dec2_up1, dec1_final. The first three have no effect for
+                                      whole events at width 16, where one kernel with one CTA
+                                      per SM runs these layers                                */
     int32_t tail_ctas_per_sm;      /* peak finder: 1..8                                         */
 } pvf_schedule;
 
@@ -213,8 +215,8 @@ PVF_API pvf_status pvf_calibrate(pvf_handle *h, const pvf_tracks_soa *tracks,
 PVF_API pvf_status pvf_last_device_status(pvf_handle *h, int32_t *out_status, pvf_stream_t stream);
 
 /* Failure detection (§3 bounds every device-side wait; the paper has no test counterpart):
- * runs the tensor-core enc2 kernel on the handle's first n_events events with its MMA
- * thread waiting, for limit_us microseconds, on a barrier that nothing arrives on. The wait
+ * runs the tensor-core encoder kernel on the handle's first n_events events with its enc2
+ * MMA warp waiting, for limit_us microseconds, on a barrier that nothing arrives on. The wait
  * gives up, the kernel raises PVF_ERR_TIMEOUT in the device status word, waits (bounded)
  * for its own copies in flight, frees its tensor memory and returns; the handle stays
  * usable. For tests of the bounded-wait path (every production wait gives up after 1 s).

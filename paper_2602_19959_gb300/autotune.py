@@ -7,7 +7,9 @@ A launch's schedule has two kinds of free parameters:
   * the grids: how many CTAs per SM each persistent kernel family launches (pvf_schedule:
     the front, whose grid sets the events each CTA walks and, in the tensor-core forms,
     the FC tile (passes of 256 tracks at 1-2 CTAs per SM, 128 at 3-4), the six tensor-core conv
-    kernels, whose grids set the tiles per CTA, and the peak finder). More resident CTAs
+    kernels, whose grids set the tiles per CTA, and the peak finder; the three encoder entries
+    act in the per-interval layout and the wide network only, where they are kernels of their
+    own). More resident CTAs
     hide latency; fewer leave each CTA more shared-memory and register headroom and
     shorten the tail of the last wave.
 For a workload the tuner captures the whole batch as one CUDA graph per candidate, times

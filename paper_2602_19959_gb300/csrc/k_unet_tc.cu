@@ -53,6 +53,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 namespace pvf {
 namespace {
@@ -237,7 +238,7 @@ template <class C> struct Bars {
     static constexpr int W = 0, FULL = 1, EMPTY = 1 + C::STAGES, TFULL = 1 + 2 * C::STAGES,
                          TEMPTY = TFULL + C::NB, T2FULL = TEMPTY + C::NB, A2FULL = T2FULL + C::NB,
                          DRAIN = A2FULL + 2, GREADY = DRAIN + 1, XREADY = GREADY + 2,
-                         TIDF = XREADY + 2, TIDE = TIDF + kRing, NEVER = TIDE + kRing, N = NEVER + 1;
+                         TIDF = XREADY + 2, TIDE = TIDF + kRing, N = TIDE + kRing;
     // after the barriers: TMEM address slot, abort flag, then the ring of tile indices
     static constexpr int RING_OFF = N * 8 + 16;
     static_assert(RING_OFF + 4 * kRing <= 512, "barrier area");
@@ -355,59 +356,55 @@ __device__ __forceinline__ void mma_t(uint32_t d, uint64_t ad, uint64_t bd, uint
     else mma_fp8(d, ad, bd, idesc, acc);
 }
 
+// The MMAs of one conv tile, from one thread. The operands lie at constant distances from the tile's and the weights' first descriptor.
 template <class C>
 __device__ __forceinline__ void issue_conv(uint32_t d, uint32_t as, uint32_t w_base) {
     if constexpr (C::PAIRED) {
         // weights: group g (taps 2g, 2g + 1; g = 2: tap 4) at w_base + g * GROUP, planes of N_g rows
         constexpr uint32_t N01 = 2 * C::COUT, GROUP = C::PIN * N01 * 16;
         constexpr uint32_t ID01 = idesc_f32acc(kTileM, N01, C::FMT), ID4 = idesc_f32acc(kTileM, C::COUT, C::FMT);
+        const uint64_t a0 = smem_desc(as, C::ROWS * 16, 128);
+        const uint64_t b0 = smem_desc(w_base, N01 * 16, 128), b4 = smem_desc(w_base + 2 * GROUP, C::COUT * 16, 128);
 #pragma unroll
         for (int kb = 0; kb < C::PIN / 2; ++kb) {
-            const uint32_t a = as + 2 * kb * C::ROWS * 16;
 #pragma unroll
             for (int g = 0; g < 2; ++g)
-                mma_t<C>(d, smem_desc(a + 2 * g * 16, C::ROWS * 16, 128),
-                         smem_desc(w_base + g * GROUP + 2 * kb * N01 * 16, N01 * 16, 128), ID01, (kb | g) != 0);
-            mma_t<C>(d, smem_desc(a + 4 * 16, C::ROWS * 16, 128),
-                     smem_desc(w_base + 2 * GROUP + 2 * kb * C::COUT * 16, C::COUT * 16, 128), ID4, true);
+                mma_t<C>(d, desc_plus(a0, 2 * kb * C::ROWS + 2 * g), desc_plus(b0, g * (GROUP / 16) + 2 * kb * N01),
+                         ID01, (kb | g) != 0);
+            mma_t<C>(d, desc_plus(a0, 2 * kb * C::ROWS + 4), desc_plus(b4, 2 * kb * C::COUT), ID4, true);
         }
     } else if constexpr (C::PAIR) {
+        const uint64_t a0 = smem_desc(as, 16, 128), b0 = smem_desc(w_base, C::COUT * 16, 128);
 #pragma unroll
-        for (int j = 0; j < C::TAPS / 2; ++j) {
-            const uint64_t ad = smem_desc(as + 2 * j * 16, 16, 128);
-            const uint64_t bd = smem_desc(w_base + 2 * j * C::COUT * 16, C::COUT * 16, 128);
-            mma_t<C>(d, ad, bd, C::IDESC1, j != 0);
-        }
+        for (int j = 0; j < C::TAPS / 2; ++j)
+            mma_t<C>(d, desc_plus(a0, 2 * j), desc_plus(b0, 2 * j * C::COUT), C::IDESC1, j != 0);
     } else {
+        const uint64_t a0 = smem_desc(as, C::ROWS * 16, 128), b0 = smem_desc(w_base, C::COUT * 16, 128);
 #pragma unroll
         for (int tap = 0; tap < C::TAPS; ++tap)
 #pragma unroll
-            for (int kb = 0; kb < C::PIN / 2; ++kb) {
-                const uint64_t ad = smem_desc(as + 2 * kb * C::ROWS * 16 + tap * 16, C::ROWS * 16, 128);
-                const uint64_t bd = smem_desc(w_base + (tap * C::PIN + 2 * kb) * C::COUT * 16,
-                                              C::COUT * 16, 128);
-                mma_t<C>(d, ad, bd, C::IDESC1, (tap | kb) != 0);
-            }
+            for (int kb = 0; kb < C::PIN / 2; ++kb)
+                mma_t<C>(d, desc_plus(a0, 2 * kb * C::ROWS + tap), desc_plus(b0, (tap * C::PIN + 2 * kb) * C::COUT),
+                         C::IDESC1, (tap | kb) != 0);
     }
 }
 
 template <class C>
 __device__ __forceinline__ void issue_up(uint32_t d2, uint32_t a2, uint32_t w2_base) {
+    const uint64_t a0 = smem_desc(a2, kTileM * 16, 128), b0 = smem_desc(w2_base, C::N2 * 16, 128);
 #pragma unroll
-    for (int kb = 0; kb < C::P2 / 2; ++kb) {
-        const uint64_t ad = smem_desc(a2 + 2 * kb * kTileM * 16, kTileM * 16, 128);
-        const uint64_t bd = smem_desc(w2_base + 2 * kb * C::N2 * 16, C::N2 * 16, 128);
-        mma_t<C>(d2, ad, bd, C::IDESC2, kb != 0);
-    }
+    for (int kb = 0; kb < C::P2 / 2; ++kb)
+        mma_t<C>(d2, desc_plus(a0, 2 * kb * kTileM), desc_plus(b0, 2 * kb * C::N2), C::IDESC2, kb != 0);
 }
 
 // The fused ConvT with its A operand in tensor memory (A2T): the K step kb reads the 8
 // columns holding channels [16 kb, 16 kb + 16) (16-bit; 32 e4m3 channels per step).
 template <class C>
 __device__ __forceinline__ void issue_up_ts(uint32_t d2, uint32_t a2_tmem, uint32_t w2_base) {
+    const uint64_t b0 = smem_desc(w2_base, C::N2 * 16, 128);
 #pragma unroll
     for (int kb = 0; kb < C::P2 / 2; ++kb) {
-        const uint64_t bd = smem_desc(w2_base + 2 * kb * C::N2 * 16, C::N2 * 16, 128);
+        const uint64_t bd = desc_plus(b0, 2 * kb * C::N2);
         if constexpr (is16(C::PREC)) mma_f16_ts(d2, a2_tmem + 8 * kb, bd, C::IDESC2, kb != 0);
         else mma_fp8_ts(d2, a2_tmem + 8 * kb, bd, C::IDESC2, kb != 0);
     }
@@ -421,9 +418,10 @@ __device__ __forceinline__ void issue_up_any(uint32_t tmem, int bp, int ap, uint
         issue_up<C>(tmem + bp * C::COLS_BUF + C::UP_OFF, a2_base + ap * C::A2_BYTES, w2_base);
 }
 
-// One thread issues all MMAs. With a fused ConvT, the conv of tile i is issued before the
-// ConvT of tile i - 1, so the tensor core works while the epilogue turns tile i - 1's
-// conv accumulator into the shared-memory operand of its ConvT.
+// One thread issues all MMAs. With a fused ConvT,
+// the conv of tile i is issued before the ConvT of tile i - 1, so the tensor core works while
+// the epilogue turns tile i - 1's conv accumulator into the operand of its ConvT. The ring
+// positions and parities are counted along instead of divided out of the tile number.
 template <class C>
 __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, uint32_t tmem,
                            volatile int *ring, volatile int *abort) {
@@ -437,20 +435,20 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
     const uint32_t w_base = smem_u32(smem + C::OFF_W);
     const uint32_t w2_base = smem_u32(smem + C::OFF_W2);
     const uint32_t a2_base = smem_u32(smem + C::OFF_A2);
-    const int ntiles = a.n_events * C::TPE;
+    const int ntiles = a.n_events * C::TPE, step = (int)gridDim.x / C::NSPLIT;
+    int s = 0, b = 0, bp = 0, r = 0;          // stage, accumulator, the previous tile's, ring slot
+    uint32_t ph_s = 0, ph_b = 0, ph_r = 0;    // their parities
     int i = 0;
-    for (; ok; ++i) {
+    for (int t = (int)blockIdx.x / C::NSPLIT; ok; ++i, t += step) {
         if constexpr (C::DYN) {
-            const int r = i % kRing;
-            if (!mbar_wait(&tidf[r], (i / kRing) & 1, abort)) { ok = false; break; }
-            const int t = ring[r];
+            if (!mbar_wait(&tidf[r], ph_r, abort)) { ok = false; break; }
+            const bool done = ring[r] < 0;
             mbar_arrive(&tide[r]);
-            if (t < 0) break;
-        } else if ((int)blockIdx.x / C::NSPLIT + i * ((int)gridDim.x / C::NSPLIT) >= ntiles) {
+            if (done) break;
+            if (++r == kRing) { r = 0; ph_r ^= 1; }
+        } else if (t >= ntiles) {
             break;
         }
-        const int s = i % C::STAGES, b = i % C::NB;
-        const uint32_t ph_s = (i / C::STAGES) & 1, ph_b = (i / C::NB) & 1;
         if (!mbar_wait(&tempty[b], ph_b ^ 1, abort) || !mbar_wait(&full[s], ph_s, abort)) { ok = false; break; }
         tc_fence_after();
         issue_conv<C>(tmem + b * C::COLS_BUF, a_base + s * C::A_STAGE, w_base);
@@ -458,17 +456,20 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
         mma_commit(&tfull[b]);
         if constexpr (C::EPI == EPI_UP) {
             if (i > 0) {
-                const int bp = (i - 1) % C::NB, ap = (i - 1) & 1;
+                const int ap = (i - 1) & 1;
                 if (!mbar_wait(&a2full[ap], ((i - 1) >> 1) & 1, abort)) { ok = false; break; }
                 tc_fence_after();
                 issue_up_any<C>(tmem, bp, ap, a2_base, w2_base);
                 mma_commit(&t2full[bp]);
             }
+            bp = b;
         }
+        if (++s == C::STAGES) { s = 0; ph_s ^= 1; }
+        if (++b == C::NB) { b = 0; ph_b ^= 1; }
     }
     if constexpr (C::EPI == EPI_UP) {
         if (ok && i > 0) {
-            const int bp = (i - 1) % C::NB, ap = (i - 1) & 1;
+            const int ap = (i - 1) & 1;
             if (mbar_wait(&a2full[ap], ((i - 1) >> 1) & 1, abort)) {
                 tc_fence_after();
                 issue_up_any<C>(tmem, bp, ap, a2_base, w2_base);
@@ -539,7 +540,11 @@ __device__ __forceinline__ bool paired_cols(uint32_t dcol, int c0, float *sx, in
         }
     }
 #pragma unroll
-    for (int j = 0; j < W; ++j) v[j] += o[j];
+    for (int j = 0; j < W; j += 2) {
+        const float2 y = __fadd2_rn(make_float2(v[j], v[j + 1]), make_float2(o[j], o[j + 1]));
+        v[j] = y.x;
+        v[j + 1] = y.y;
+    }
     return true;
 }
 
@@ -550,7 +555,10 @@ __device__ __forceinline__ bool paired_cols(uint32_t dcol, int c0, float *sx, in
 // per-interval layout, stored as zeros). Paired taps: the exchange of each column chunk
 // meets on xready, which completed xuse0 times before this tile (returns false on a
 // timed-out wait).
-template <class C, int NC>
+// CAL: a calibration pass, which also records the largest stored magnitudes (its code, in every
+// 16-column block, stays out of the kernels that serve: they would not fit the instruction
+// cache as well).
+template <class C, int NC, bool CAL, int LDW = C::ldw(NC)>
 __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, const float *sbias,
                                          const float *scs, uint32_t dcol, int c_beg, int ab, int e,
                                          int p, int m, bool valid, float *sx = nullptr,
@@ -561,7 +569,6 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
     seq_pos<C>(p, sq, jq);
     // pooled row: position j / 2 of sequence s (whole events: p / 2)
     const int64_t prow = C::SEQ ? (int64_t)sq * C::SEQP + jq / 2 + kPad : p / 2 + kPad;
-    constexpr int LDW = C::ldw(NC);
 #pragma unroll 1
     for (int cc = 0; cc < NC; cc += LDW) {
         float vv[LDW];
@@ -579,14 +586,14 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
             const int c0 = c_beg + cc + 16 * h;
             float v[16], bj[16];
             lds16(sbias + c0, bj);
-            if constexpr (is16(C::PREC)) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = leaky(vv[16 * h + j] + bj[j]);
+            for (int j = 0; j < 16; ++j) v[j] = vv[16 * h + j];
+            if constexpr (is16(C::PREC)) {
+                bias_leaky(v, bj);
             } else {
                 float sc[16];
                 lds16(scs + c0, sc);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = leaky(fmaf(vv[16 * h + j], sc[j], bj[j]));
+                scale_bias_leaky(v, sc, bj);
             }
             if constexpr (C::SEQ != 0) {
                 if (!inseq) {
@@ -597,7 +604,7 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
             if constexpr (C::EPI == EPI_UP && C::A2T) {
                 // this row's 16 channels into its TMEM lane: 16-bit pairs (8 columns) or
                 // e4m3 quads (4 columns), the K order the MMA reads
-                if (a.amax) amax_fold(a.amax, a.amax_mid, v, valid);
+                if constexpr (CAL) amax_fold(a.amax, a.amax_mid, v, valid);
                 if constexpr (is16(C::PREC)) {
                     using T = typename Elem<C::PREC>::T;
                     uint32_t r[8];
@@ -610,22 +617,48 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
                     tmem_st<4>(a2t + c0 / 4, r);
                 }
             } else if constexpr (C::EPI == EPI_UP) {
-                if (a.amax) amax_fold(a.amax, a.amax_mid, v, valid);
+                if constexpr (CAL) amax_fold(a.amax, a.amax_mid, v, valid);
                 unsigned char *a2 = smem + C::OFF_A2 + ab * C::A2_BYTES;
                 put16<C::PREC>(a2 + ((c0 / C::PW) * kTileM + m) * 16, (size_t)kTileM * 16, v, a.mid_inv);
             } else {
-                if (a.amax) amax_fold(a.amax, a.amax_out, v, valid);
-                if (valid)   // a split layer's part writes its own planes of the output
-                    put16<C::PREC>(a.out + planar_off(e, ((int)blockIdx.x % C::NSPLIT) * C::POUT + c0 / C::PW,
-                                                      C::POUT_TOT, C::ROWS_E, p + kPad),
-                              (size_t)C::ROWS_E * 16, v, a.out_inv);
-                if constexpr (C::EPI == EPI_POOL) {
-                    float w[16];
+                if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid);
+                unsigned char *dst = a.out + planar_off(e, ((int)blockIdx.x % C::NSPLIT) * C::POUT + c0 / C::PW,
+                                                        C::POUT_TOT, C::ROWS_E, p + kPad);
+                if constexpr (is16(C::PREC)) {
+                    using T = typename Elem<C::PREC>::T;
+                    uint32_t r[8];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) w[j] = fmaxf(v[j], __shfl_xor_sync(0xffffffffu, v[j], 1));
-                    if (valid && inseq && (m & 1) == 0)
-                        put16<C::PREC>(a.outp + planar_off(e, c0 / C::PW, C::POUT, ROWS_P, prow),
-                                  (size_t)ROWS_P * 16, w, a.out_inv);
+                    for (int j = 0; j < 8; ++j) r[j] = pack2<T>(v[2 * j], v[2 * j + 1]);
+                    if (valid) {   // a split layer's part writes its own planes of the output
+                        *reinterpret_cast<uint4 *>(dst) = make_uint4(r[0], r[1], r[2], r[3]);
+                        *reinterpret_cast<uint4 *>(dst + (size_t)C::ROWS_E * 16) = make_uint4(r[4], r[5], r[6], r[7]);
+                    }
+                    if constexpr (C::EPI == EPI_POOL) {
+                        // the maximum of the rounded values is the rounded maximum, so the pair of rows
+                        // exchanges its packed halves: the even row takes the first 8 channels of both
+                        // rows and stores the first plane, the odd row the last 8 and the second plane
+                        const bool odd = (m & 1) != 0;
+                        uint32_t w[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? r[j] : r[4 + j], 1);
+                            w[j] = max2<T>(odd ? r[4 + j] : r[j], got);
+                        }
+                        if (valid && inseq)
+                            *reinterpret_cast<uint4 *>(a.outp + planar_off(e, c0 / C::PW + (odd ? 1 : 0), C::POUT,
+                                                                           ROWS_P, prow)) =
+                                make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                } else {
+                    if (valid) put16<C::PREC>(dst, (size_t)C::ROWS_E * 16, v, a.out_inv);
+                    if constexpr (C::EPI == EPI_POOL) {
+                        float w[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) w[j] = fmaxf(v[j], __shfl_xor_sync(0xffffffffu, v[j], 1));
+                        if (valid && inseq && (m & 1) == 0)
+                            put16<C::PREC>(a.outp + planar_off(e, c0 / C::PW, C::POUT, ROWS_P, prow),
+                                           (size_t)ROWS_P * 16, w, a.out_inv);
+                    }
                 }
             }
         }
@@ -636,7 +669,7 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
 // Fused ConvT columns [n_beg, n_beg + NC) (n = r * CUP + co: output row 2p + r, channel
 // co): bias, LeakyReLU, store; the thread of p = 0 / L - 1 (with pads) zeroes the pads.
 // r0: the first output-row parity of these columns (the ConvT GEMM split by r: its part).
-template <class C, int NC>
+template <class C, int NC, bool CAL, int LDW = NC % 32 == 0 ? 32 : 16>
 __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, const float *scs2,
                                        uint32_t dcol, int n_beg, int e, int p, bool valid, bool pads,
                                        int r0 = 0) {
@@ -648,7 +681,6 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
     // output rows 2 j + r of sequence s (whole events: 2 p + r)
     const int64_t orow0 = C::SEQ ? (int64_t)sq * C::SEQU + 2 * jq + kPad : 2 * p + kPad;
     constexpr int PUP = C::CUP / C::PW;
-    constexpr int LDW = NC % 32 == 0 ? 32 : 16;
 #pragma unroll 1
     for (int cc = 0; cc < NC; cc += LDW) {
         float vv[LDW];
@@ -663,16 +695,16 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
             const int r = r0 + c0 / C::CUP, co0 = c0 % C::CUP;
             float v[16], bj[16];
             lds16(sbias2 + co0, bj);
-            if constexpr (is16(C::PREC)) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = leaky(vv[16 * h + j] + bj[j]);
+            for (int j = 0; j < 16; ++j) v[j] = vv[16 * h + j];
+            if constexpr (is16(C::PREC)) {
+                bias_leaky(v, bj);
             } else {
                 float sc[16];
                 lds16(scs2 + c0, sc);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = leaky(fmaf(vv[16 * h + j], sc[j], bj[j]));
+                scale_bias_leaky(v, sc, bj);
             }
-            if (a.amax) amax_fold(a.amax, a.amax_out, v, valid && inseq);
+            if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid && inseq);
             if (valid && inseq)
                 put16<C::PREC>(a.out + planar_off(e, co0 / C::PW, PUP, ROWS_O, orow0 + r),
                           (size_t)ROWS_O * 16, v, a.out_inv);
@@ -699,7 +731,7 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
     }
 }
 
-template <class C>
+template <class C, bool CAL>
 __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, uint32_t tmem,
                          volatile int *ring, volatile int *abort, int warp, int lane) {
     using B = Bars<C>;
@@ -748,7 +780,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             if (wg < PER) {     // conv accumulator -> ConvT operand
                 if (!mbar_wait(&tfull[b], ph_b, abort)) return false;
                 tc_fence_after();
-                if (!epi_conv<C, C::COUT / PER>(a, smem, sbias, scs, dcol, part * (C::COUT / PER), ab, e, p, m,
+                if (!epi_conv<C, C::COUT / PER, CAL>(a, smem, sbias, scs, dcol, part * (C::COUT / PER), ab, e, p, m,
                                                 valid, sx, a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
                                                 (uint32_t)(i >> 1) * C::xchunks(C::COUT / PER), abort))
                     return false;
@@ -759,7 +791,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             } else {            // ConvT accumulator -> output; frees the buffer
                 if (!mbar_wait(&t2full[b], ph_b, abort)) return false;
                 tc_fence_after();
-                epi_up<C, C::N2 / PER>(a, sbias2, scs2, dcol, part * (C::N2 / PER), e, p, valid, part == 0);
+                epi_up<C, C::N2 / PER, CAL>(a, sbias2, scs2, dcol, part * (C::N2 / PER), e, p, valid, part == 0);
                 tc_fence_before();
                 mbar_arrive(&tempty[b]);
             }
@@ -768,7 +800,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
         if (!mbar_wait(&tfull[b], ph_b, abort)) return false;
         tc_fence_after();
         if constexpr (C::EPI == EPI_CONVT) {   // the ConvT GEMM: this warpgroup's columns
-            epi_up<C, C::EPI_COLS>(a, sbias, scs, dcol, wg * C::EPI_COLS, e, p, valid, wg == 0 && part == 0,
+            epi_up<C, C::EPI_COLS, CAL>(a, sbias, scs, dcol, wg * C::EPI_COLS, e, p, valid, wg == 0 && part == 0,
                                    part * (C::COUT / C::CUP));
             tc_fence_before();
             mbar_arrive(&tempty[b]);
@@ -791,16 +823,14 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             for (int ch = 0; ch < NCH; ++ch) {
                 float bj[16], sc[16];
                 lds16(sbias + 16 * ch, bj);
-                if constexpr (is16(C::PREC)) {
+                if constexpr (!is16(C::PREC)) lds16(scs + 16 * ch, sc);
+                if constexpr (is16(C::PREC)) bias_leaky(v[ch], bj);
+                else scale_bias_leaky(v[ch], sc, bj);
+                if (!(valid && inseq)) {   // zero padding outside the event or its sequence
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) sc[j] = 1.0f;
-                } else {
-                    lds16(scs + 16 * ch, sc);
+                    for (int j = 0; j < 16; ++j) v[ch][j] = 0.0f;
                 }
-#pragma unroll
-                for (int j = 0; j < 16; ++j)   // zero padding outside the event or its sequence
-                    v[ch][j] = valid && inseq ? leaky(fmaf(v[ch][j], sc[j], bj[j])) : 0.0f;
-                if (a.amax) amax_fold(a.amax, a.amax_out, v[ch], valid && inseq);
+                if constexpr (CAL) amax_fold(a.amax, a.amax_out, v[ch], valid && inseq);
                 // the final conv's partial sums over this chunk's channels, in channel order:
                 // taps (0, 1) and (2, 3) as packed two-lane FMAs (each lane an fmaf), from
                 // weights stored per channel as (w0, w1, w2, w3), then tap 4
@@ -842,7 +872,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             continue;
         }
         if constexpr (C::EPI == EPI_UP) {   // one warpgroup: conv, then the ConvT
-            if (!epi_conv<C, C::COUT>(a, smem, sbias, scs, dcol, 0, ab, e, p, m, valid, sx,
+            if (!epi_conv<C, C::COUT, CAL>(a, smem, sbias, scs, dcol, 0, ab, e, p, m, valid, sx,
                                       a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
                                       (uint32_t)(i >> 1) * C::xchunks(C::COUT), abort))
                 return false;
@@ -852,11 +882,11 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             mbar_arrive(&a2full[ab]);
             if (!mbar_wait(&t2full[b], ph_b, abort)) return false;
             tc_fence_after();
-            epi_up<C, C::N2>(a, sbias2, scs2, dcol, 0, e, p, valid, true);
+            epi_up<C, C::N2, CAL>(a, sbias2, scs2, dcol, 0, e, p, valid, true);
         } else {                            // this warpgroup's conv columns
             static_assert(!C::PAIRED || C::EPI == EPI_STORE, "paired stores");
             // paired taps (the wide network's split dec3): E[m] + O[m + 1]
-            if (!epi_conv<C, C::EPI_COLS>(a, smem, sbias, scs, dcol, wg * C::EPI_COLS, ab, e, p, m, valid, sx, 0,
+            if (!epi_conv<C, C::EPI_COLS, CAL>(a, smem, sbias, scs, dcol, wg * C::EPI_COLS, ab, e, p, m, valid, sx, 0,
                                           inseq, &xready[ab], (uint32_t)(i >> 1) * C::xchunks(C::EPI_COLS), abort))
                 return false;
             if (wg == 0 && (p == 0 || p == C::L - 1)) {
@@ -884,7 +914,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
     return true;
 }
 
-template <class C>
+template <class C, bool CAL>
 __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(TcArgs a) {
     using B = Bars<C>;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -930,7 +960,6 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
             mbar_init(&bar[B::TIDF + r], 1);                // the producer
             mbar_init(&bar[B::TIDE + r], 1 + 4 * C::EWG);   // the MMA thread and each epilogue warp
         }
-        mbar_init(&bar[B::NEVER], 1);                       // bounded-wait tests: nobody arrives
         *abort = 0;
         fence_mbar_init();
     }
@@ -954,12 +983,13 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
     if (warp == 0) {
         if (lane == 0) ok = producer<C>(r, smem, bar, ring, abort);
     } else if (warp == 1) {
-        // a test of the bounded waits: the wait gives up after stall_test_us, before any MMA
-        if (lane == 0 && a.stall_test_us)
-            ok = mbar_wait(&bar[B::NEVER], 0, abort, 1000ull * a.stall_test_us);
-        if (lane == 0 && ok) ok = mma_issuer<C>(r, smem, bar, tmem, ring, abort);
+        // The split layers' CTAs, which only convolve and store, gain from MMAs issued at the
+        // elected thread's rate (wide dec3 107 -> 94 us, enc4 49 -> 42 per 250 events); where the
+        // epilogues share the SM with a second GEMM or a pool the same rate costs (dec3_up2 94 ->
+        // 97 us per 1000 events, FP8 dec2_up1 57 -> 60): they keep the plain one-thread branch.
+        if (C::NSPLIT > 1 ? elect_one() : lane == 0) ok = mma_issuer<C>(r, smem, bar, tmem, ring, abort);
     } else {
-        ok = epilogue<C>(r, smem, bar, tmem, ring, abort, warp, lane);
+        ok = epilogue<C, CAL>(r, smem, bar, tmem, ring, abort, warp, lane);
     }
     if (!ok) {
         *abort = 1;
@@ -979,8 +1009,10 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
 }
 
 // cap: the launch schedule's CTAs per SM (0 = as many as fit)
-template <class C>
+template <class C, bool CAL = false>
 cudaError_t launch_conv(const TcArgs &a, cudaStream_t s, const ProfHook *prof, const char *name, int cap) {
+    if constexpr (C::PREC == PVF_BF16 && !CAL)
+        if (a.amax) return launch_conv<C, true>(a, s, prof, name, cap);      // calibration runs in the BF16 form
     if (a.n_events <= 0) return cudaSuccess;
     // shared memory request padded so that the CTAs resident on one SM never ask for more
     // than the 512 TMEM columns: tcgen05.alloc would otherwise wait for a neighbour
@@ -993,7 +1025,7 @@ cudaError_t launch_conv(const TcArgs &a, cudaStream_t s, const ProfHook *prof, c
     int sms = 0;
     cudaFuncAttributes fa;
     cudaError_t err = current_device_sms(&sms);
-    if (err == cudaSuccess) err = prepare_kernel((const void *)k_conv_tc<C>, (size_t)smem, &fa);
+    if (err == cudaSuccess) err = prepare_kernel((const void *)k_conv_tc<C, CAL>, (size_t)smem, &fa);
     if (err != cudaSuccess) return err;
     // resident CTAs per SM: registers (each of the 4 sub-partitions holds 16K, allocated
     // per warp in units of 256), shared memory (+1 KB reserved per CTA), threads, TMEM
@@ -1012,7 +1044,7 @@ cudaError_t launch_conv(const TcArgs &a, cudaStream_t s, const ProfHook *prof, c
     grid = grid / C::NSPLIT * C::NSPLIT;             // every part gets the same CTAs
     if (grid < C::NSPLIT) grid = C::NSPLIT;
     ProfScope ps(prof, name, s);
-    return launch_pdl(k_conv_tc<C>, dim3(grid), dim3(C::THREADS), (size_t)smem, s, a);
+    return launch_pdl(k_conv_tc<C, CAL>, dim3(grid), dim3(C::THREADS), (size_t)smem, s, a);
 }
 
 // ---------------------------------------------------------------- weight packing (host)
@@ -1024,6 +1056,7 @@ cudaError_t launch_conv(const TcArgs &a, cudaStream_t s, const ProfHook *prof, c
 constexpr bool conv_paired(int li, int prec) { return (li == 3 || li == 4) && is16(prec); }
 
 template <int PREC> struct Net {
+    static constexpr bool FUSED_ENC = true;    // enc2, enc3 and enc4 + up3 run as k_enc_tc
     using Enc2 = Cfg<PREC, 16, 0, 32, 2000, EPI_POOL, 0, 4, 1, 56, 2, false, true>;    // 6 CTAs per SM
     using Enc3 = Cfg<PREC, 32, 0, 64, 1000, EPI_POOL, 0, 4, 1, 80, 2, false, true>;    // 4
     // the fused-ConvT kernels keep the ConvT operand in TMEM (three accumulator buffers
@@ -1032,7 +1065,7 @@ template <int PREC> struct Net {
                         is16(PREC) ? 2 : 4, 96, 3, false, false, true>;              // 1
     using Dec3Up2 = Cfg<PREC, 64, 64, 64, 1000, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false,
                         true>;                                                         // 1 CTA/SM
-    using Dec2Up1 = Cfg<PREC, 32, 32, 32, 2000, EPI_UP, 16, 3, 2, 128, 3, conv_paired(4, PREC), false,
+    using Dec2Up1 = Cfg<PREC, 32, 32, 32, 2000, EPI_UP, 16, 3, 2, 96, 3, conv_paired(4, PREC), false,
                         true>;                                                         // 2
     using Dec1Final = Cfg<PREC, 16, 16, 16, 4000, EPI_FINAL, 0, 3, 1, 64, 4, conv_paired(5, PREC)>; // 5
 };
@@ -1041,6 +1074,7 @@ template <int PREC> struct Net {
 // 104 positions): the same kernels over each event's 40 sequences laid end to end, with
 // levels of 104, 52, 26 and 13 positions per sequence (108, 56, 30 and 17 storage rows).
 template <int PREC> struct NetIv {
+    static constexpr bool FUSED_ENC = false;   // the pooled rows of its sequences do not tile 2 : 1
     static constexpr int S0 = kIvLen + kPad, S1 = kIvLen / 2 + kPad, S2 = kIvLen / 4 + kPad,
                          S3 = kIvLen / 8 + kPad;
     static constexpr int L0 = kSlices * S0 - kPad, L1 = kSlices * S1 - kPad, L2 = kSlices * S2 - kPad,
@@ -1054,6 +1088,8 @@ template <int PREC> struct NetIv {
     using Dec1Final = Cfg<PREC, 16, 16, 16, L0, EPI_FINAL, 0, 3, 1, 64, 4, conv_paired(5, PREC), false, false,
                           S0>;
 };
+
+#include "enc_tc.cuh"
 
 // The wide network (base width 32: 32/64/128/256 channels, §5's channel-count axis). The
 // enc4 (128 -> 256) and dec3 (256 -> 128) weight images (320 KB in 16 bits) exceed a CTA's
@@ -1270,18 +1306,26 @@ static cudaError_t run_tc(const TcNet &n, const UnetBuffers &b, int ne, const in
     auto sched = [&](int k) { return n.sched + 2 * k; };
     a.sched = sched(0);
     // enc2: p1 (s0) -> e2, p2 (s1)
+    EncArgs g;
     a.inA = U(b.s0); a.inB = nullptr; a.out = U(b.e2); a.outp = U(b.s1);
     a.w = W(0); a.bias = n.b[0]; a.cs = cs(0); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
-    if ((err = launch_conv<typename N::Enc2>(a, s, prof, "enc2", n.ctas_per_sm[0])) != cudaSuccess) return err;
+    if constexpr (N::FUSED_ENC) g.c2 = a;
+    else if ((err = launch_conv<typename N::Enc2>(a, s, prof, "enc2", n.ctas_per_sm[0])) != cudaSuccess) return err;
     // enc3: p2 (s1) -> e3, p3 (s0)
     a.inA = U(b.s1); a.out = U(b.e3); a.outp = U(b.s0); a.sched = sched(1);
     a.w = W(1); a.bias = n.b[1]; a.cs = cs(1); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
-    if ((err = launch_conv<typename N::Enc3>(a, s, prof, "enc3", n.ctas_per_sm[1])) != cudaSuccess) return err;
+    if constexpr (N::FUSED_ENC) g.c3 = a;
+    else if ((err = launch_conv<typename N::Enc3>(a, s, prof, "enc3", n.ctas_per_sm[1])) != cudaSuccess) return err;
     // enc4 + up3: p3 (s0) -> u3 (up)
     a.inA = U(b.s0); a.out = U(b.up); a.outp = nullptr; a.sched = sched(2);
     a.w = W(2); a.bias = n.b[2]; a.cs = cs(2); a.w2 = W(6); a.bias2 = n.b[6]; a.cs2 = cs(6);
     a.mid_inv = inv(kScaleE4); a.out_inv = inv(kScaleL3); a.amax_mid = kScaleE4; a.amax_out = kScaleL3;
-    if ((err = launch_conv<typename N::Enc4Up3>(a, s, prof, "enc4_up3", n.ctas_per_sm[2])) != cudaSuccess) return err;
+    if constexpr (N::FUSED_ENC) {      // the three layers in one kernel; p2 and p3 stay in shared memory
+        g.c4 = a;
+        if ((err = launch_enc<N>(g, s, prof)) != cudaSuccess) return err;
+    } else if ((err = launch_conv<typename N::Enc4Up3>(a, s, prof, "enc4_up3", n.ctas_per_sm[2])) != cudaSuccess) {
+        return err;
+    }
     // dec3 + up2: [u3 (up), e3] -> u2 (deep)
     a.inA = U(b.up); a.inB = U(b.e3); a.out = U(b.deep); a.sched = sched(3);
     a.w = W(3); a.bias = n.b[3]; a.cs = cs(3); a.w2 = W(7); a.bias2 = n.b[7]; a.cs2 = cs(7);
@@ -1356,7 +1400,7 @@ static cudaError_t run_tc32(const TcNet &n, const UnetBuffers &b, int ne, const 
     return launch_conv<typename N::Dec1Final>(a, s, prof, "dec1_final", n.ctas_per_sm[5]);
 }
 
-// The enc2 kernel alone with its MMA thread stalled for stall_us (tests of the bounded waits).
+// The encoder kernel alone with its enc2 MMA warp stalled for stall_us (tests of the bounded waits).
 template <int PREC>
 static cudaError_t stall_tc(const TcNet &n, const UnetBuffers &b, int ne, uint32_t stall_us, cudaStream_t s) {
     using N = Net<PREC>;
@@ -1372,7 +1416,15 @@ static cudaError_t stall_tc(const TcNet &n, const UnetBuffers &b, int ne, uint32
     a.cs = is16(PREC) ? nullptr : n.wscale[0];
     a.out_inv = is16(PREC) ? 1.0f : 1.0f / n.act_scale[kScaleL2];
     a.stall_test_us = stall_us;
-    return launch_conv<typename N::Enc2>(a, s, nullptr, "enc2", n.ctas_per_sm[0]);
+    EncArgs g;
+    g.c2 = g.c3 = g.c4 = a;
+    g.c3.w = static_cast<const unsigned char *>(n.w[1]);
+    g.c3.bias = n.b[1];
+    g.c4.w = static_cast<const unsigned char *>(n.w[2]);
+    g.c4.bias = n.b[2];
+    g.c4.w2 = static_cast<const unsigned char *>(n.w[6]);
+    g.c4.bias2 = n.b[6];
+    return launch_enc<N>(g, s, nullptr);
 }
 
 cudaError_t launch_stall_test_tc(const TcNet &net, const UnetBuffers &b, int n, uint32_t stall_us,

@@ -68,6 +68,38 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
+// The same operations on 32-bit shared-memory addresses, for code that keeps them in registers
+// (a 64-bit generic pointer that may be null, or is chosen at run time, costs a conversion per
+// use and generic instead of shared accesses).
+__device__ __forceinline__ void mbar_arrive_at(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ void sts16(uint32_t a, uint4 v) {
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void sts8(uint32_t a, uint2 v) {
+    asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+// 16 floats at a 16-byte aligned shared address that the kernel's prologue filled.
+__device__ __forceinline__ void lds16_at(uint32_t a, float (&v)[16]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+            : "=f"(v[4 * i]), "=f"(v[4 * i + 1]), "=f"(v[4 * i + 2]), "=f"(v[4 * i + 3])
+            : "r"(a + 16 * i));
+}
+
 // Longest any wait may take before the kernel gives up (1 s).
 constexpr uint64_t kWaitLimitNs = 1000000000ull;
 
@@ -84,6 +116,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
             if (*abort) return false;
             if (globaltimer() - t0 > limit_ns) return false;
         }
+    }
+}
+
+__device__ __forceinline__ bool mbar_wait_at(uint32_t bar, uint32_t parity, volatile int *abort) {
+    if (mbar_try_wait_at(bar, parity)) return true;
+    const uint64_t t0 = globaltimer();
+    for (uint32_t it = 1;; ++it) {
+        if (mbar_try_wait_at(bar, parity)) return true;
+        if ((it & 255) == 0 && (*abort || globaltimer() - t0 > kWaitLimitNs)) return false;
+    }
+}
+
+// The same wait by all 32 threads of a warp; the result is the same in every thread (a vote),
+// so the code after it stays warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort,
+                                               uint64_t limit_ns = kWaitLimitNs) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const uint64_t t0 = globaltimer();
+    for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((it & 255) == 0 && __any_sync(0xffffffffu, *abort || globaltimer() - t0 > limit_ns)) return false;
     }
 }
 
@@ -137,6 +190,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return d;
 }
 
+// The descriptor of the operand `rows16` 16-byte units further on (the address field does not
+// overflow: shared memory ends below 2^18 bytes).
+__device__ __forceinline__ uint64_t desc_plus(uint64_t d, uint32_t units16) {
+    return (d & 0xFFFFFFFF00000000ull) | (uint32_t)((uint32_t)d + units16);
+}
+
 // Instruction descriptor of tcgen05.mma: D f32, A/B K-major, dense.
 //   kind::f16     a/b format 0 = f16, 1 = bf16 (A and B always of the same type)
 //   kind::f8f6f4  a/b format 0 = e4m3
@@ -146,6 +205,9 @@ __host__ __device__ constexpr uint32_t idesc_f32acc(int M, int N, uint32_t ab_fo
 }
 
 // ------------------------------------------------------------------ MMA
+//
+// One thread issues them: the waits around a tile's MMAs are the whole warp's, the MMAs and
+// their commits stand in one branch that elect_one() opens.
 
 // kind::f16: bf16 or f16 operands, as the instruction descriptor says
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
@@ -185,6 +247,15 @@ __device__ __forceinline__ void mma_fp8_ts(uint32_t d_tmem, uint32_t a_tmem, uin
         "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+
+// True in one thread of the warp, the same one at every call (all 32 threads call it).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok));
+    return ok != 0;
 }
 
 // Arrives on `bar` once every MMA issued so far by this thread has completed.
