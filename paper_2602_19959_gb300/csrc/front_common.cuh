@@ -38,6 +38,29 @@ __device__ __forceinline__ void store_row16(void *base, int64_t e, int64_t rows_
     }
 }
 
+// Channels [16 g, 16 g + 16) of position p of event e in a quad-layout tensor of C0 channels
+// and `rows` rows per residue plane.
+template <class T, int C0>
+__device__ __forceinline__ void store_seg16_quad(void *base, int64_t e, int rows, int p, int g, const float v[16],
+                                                 float inv_scale) {
+    unsigned char *cb = reinterpret_cast<unsigned char *>(base);
+    if constexpr (sizeof(T) == 2) {
+        *reinterpret_cast<uint4 *>(cb + quad_off(e, 2 * g, C0 / 8, rows, p)) = pack8<T>(v);
+        *reinterpret_cast<uint4 *>(cb + quad_off(e, 2 * g + 1, C0 / 8, rows, p)) = pack8<T>(v + 8);
+    } else {
+        uint4 pk;
+        pack_e4m3<16>(v, inv_scale, reinterpret_cast<uint32_t *>(&pk));
+        *reinterpret_cast<uint4 *>(cb + quad_off(e, g, C0 / 16, rows, p)) = pk;
+    }
+}
+// All channels of position p set to zero.
+template <class T, int C0> __device__ __forceinline__ void zero_quad(void *base, int64_t e, int rows, int p) {
+    unsigned char *cb = reinterpret_cast<unsigned char *>(base);
+    constexpr int P = C0 * (int)sizeof(T) / 16;
+#pragma unroll
+    for (int k = 0; k < P; ++k) *reinterpret_cast<uint4 *>(cb + quad_off(e, k, P, rows, p)) = make_uint4(0, 0, 0, 0);
+}
+
 // Channels [16 g, 16 g + 16) of storage row `row` of event e in a plane-major tensor of C0
 // channels (16-bit: planes 2 g and 2 g + 1 of C0 / 8; e4m3: plane g of C0 / 16).
 template <class T, int C0>
@@ -213,7 +236,7 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
                                             const float *senc) {
     static_assert(NT % 2 == 0, "thread pairs");
     constexpr int S1 = kIvLen + kPad, S2 = kIvLen / 2 + kPad;   // rows per sequence
-    const int64_t rows1 = IV ? (int64_t)kSlices * S1 + kPad : padded_rows(kBins);
+    constexpr int RQ = quad_rows(IV ? kSlices * S1 - kPad : kBins);     // e1: the quad layout
     const int64_t rows2 = IV ? (int64_t)kSlices * S2 + kPad : padded_rows(kBins / 2);
     constexpr int NQ = IV ? kSlices * (kIvLen / 2) : kBins / 2;         // position pairs
     const float inv = a.e1_inv_scale;
@@ -228,9 +251,10 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
     float vmax = 0.0f;
 #pragma unroll 2   // two position pairs in flight per thread: front 81.6 -> 79.5 us (FP16)
     for (int qi = tid >> 1; qi < NQ; qi += NT / 2) {
-        // the pair's sequence (IV) and first position; e1 rows r1, r1 + 1, p1 row r2
+        // the pair's sequence (IV) and first position; e1 positions p1, p1 + 1, p1 row r2
         const int sq = IV ? qi / (kIvLen / 2) : 0, q = IV ? qi % (kIvLen / 2) : qi;
-        const int64_t r1 = (int64_t)sq * S1 * IV + 2 * q + kPad, r2 = (int64_t)sq * S2 * IV + q + kPad;
+        const int p1 = sq * S1 * IV + 2 * q;
+        const int64_t r2 = (int64_t)sq * S2 * IV + q + kPad;
         float hv[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -267,17 +291,21 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
             // the pooled row from the packed rows: the maximum of the rounded values is the
             // rounded maximum
             const uint4 r0 = pack8<T>(v0), r1v = pack8<T>(v1);
-            unsigned char *d1 = reinterpret_cast<unsigned char *>(a.e1) + planar_off(e, h, 2, rows1, r1);
+            unsigned char *d1 = reinterpret_cast<unsigned char *>(a.e1) + quad_off(e, h, 2, RQ, p1);
             *reinterpret_cast<uint4 *>(d1) = r0;
-            *reinterpret_cast<uint4 *>(d1 + 16) = r1v;
+            *reinterpret_cast<uint4 *>(d1 + RQ * 16) = r1v;       // the next residue: p1 is even
             *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.p1) + planar_off(e, h, 2, rows2, r2)) =
                 make_uint4(max2<T>(r0.x, r1v.x), max2<T>(r0.y, r1v.y), max2<T>(r0.z, r1v.z), max2<T>(r0.w, r1v.w));
         } else {
             float vp[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) vp[j] = fmaxf(v0[j], v1[j]);
-            store_half8<T>(a.e1, e, rows1, r1, h, v0, inv);
-            store_half8<T>(a.e1, e, rows1, r1 + 1, h, v1, inv);
+            unsigned char *d1 = reinterpret_cast<unsigned char *>(a.e1) + quad_off(e, 0, 1, RQ, p1) + 8 * h;
+            uint2 pk;
+            pack_e4m3<8>(v0, inv, reinterpret_cast<uint32_t *>(&pk));
+            *reinterpret_cast<uint2 *>(d1) = pk;
+            pack_e4m3<8>(v1, inv, reinterpret_cast<uint32_t *>(&pk));
+            *reinterpret_cast<uint2 *>(d1 + RQ * 16) = pk;
             store_half8<T>(a.p1, e, rows2, r2, h, vp, inv);
         }
     }
@@ -289,12 +317,11 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
     if constexpr (IV) {     // the two rows before each sequence and the two after the last
         for (int idx = tid; idx < (kSlices + 1) * 2; idx += NT) {
             const int sq = idx >> 1, k = idx & 1;
-            zero_row16<T>(a.e1, e, rows1, (int64_t)sq * S1 + k);
+            zero_quad<T, kC0>(a.e1, e, RQ, sq * S1 + k - kPad);
             zero_row16<T>(a.p1, e, rows2, (int64_t)sq * S2 + k);
         }
     } else if (tid < 4) {
-        const int r = tid < 2 ? tid : kBins + tid;             // rows 0,1 and L+2, L+3
-        zero_row16<T>(a.e1, e, rows1, r);
+        zero_quad<T, kC0>(a.e1, e, RQ, tid < 2 ? tid - kPad : kBins + tid - kPad);   // -2, -1 and L, L + 1
         const int rp = tid < 2 ? tid : kBins / 2 + tid;
         zero_row16<T>(a.p1, e, rows2, rp);
     }
@@ -354,8 +381,8 @@ __device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, in
                 store_seg16_f32<C0>(a.e1, e, rows1, 2 * q + 1 + kPad, g, v1);
                 store_seg16_f32<C0>(a.p1, e, rows2, q + kPad, g, vp);
             } else {   // the wide network in the tensor-core forms: plane-major segments
-                store_seg16_pm<T, C0>(a.e1, e, rows1, 2 * q + kPad, g, v0, inv);
-                store_seg16_pm<T, C0>(a.e1, e, rows1, 2 * q + 1 + kPad, g, v1, inv);
+                store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), 2 * q, g, v0, inv);
+                store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), 2 * q + 1, g, v1, inv);
                 store_seg16_pm<T, C0>(a.p1, e, rows2, q + kPad, g, vp, inv);
             }
         }
@@ -380,7 +407,7 @@ __device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, in
                     store_seg16_f32<C0>(a.e1, e, rows1, r, g, z);
                     store_seg16_f32<C0>(a.p1, e, rows2, rp, g, z);
                 } else {
-                    store_seg16_pm<T, C0>(a.e1, e, rows1, r, g, z, 1.0f);
+                    store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), r - kPad, g, z, 1.0f);
                     store_seg16_pm<T, C0>(a.p1, e, rows2, rp, g, z, 1.0f);
                 }
             }

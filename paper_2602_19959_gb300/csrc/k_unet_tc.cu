@@ -10,7 +10,7 @@
 //   enc4_up3  conv 64->128 @500,  epilogue feeds a second GEMM: ConvT 128->64 (k2 s2)
 //   dec3_up2  conv [64|64]->64 @1000, + ConvT 64->32
 //   dec2_up1  conv [32|32]->32 @2000, + ConvT 32->16
-//   dec1      conv [16|16]->16 @4000, + the final conv 16->1 (logits)
+//   dec1      conv [16|16]->16 @4000, + the final conv 16->1 (logits): dec1_tc.cuh
 // The skip concat is never materialised: the two inputs are copied into adjacent
 // K-planes of the same shared-memory tile. Every conv and ConvT output goes through
 // LeakyReLU(0.01) in the epilogue; the fused ConvT reads the conv tile from shared
@@ -64,7 +64,7 @@ constexpr int kTileM = 128;
 
 // EPI_CONVT: the kernel's GEMM is itself a ConvT k2 s2 (one "tap", N = r * CUP + co), for
 // the wide network's layers whose conv is split over CTAs and so cannot fuse its ConvT.
-enum { EPI_STORE = 0, EPI_POOL = 1, EPI_UP = 2, EPI_FINAL = 3, EPI_CONVT = 4 };
+enum { EPI_STORE = 0, EPI_POOL = 1, EPI_UP = 2, EPI_CONVT = 3 };
 
 __host__ __device__ constexpr int pow2ceil(int x) {
     int p = 32;
@@ -122,11 +122,13 @@ struct Cfg {
     static constexpr int SEQU = SEQ ? 2 * LSEQ + kPad : 0;   // after the ConvT
     static constexpr int64_t ROWS_P = SEQ ? (int64_t)kSlices * SEQP + kPad : L_ / 2 + 2 * kPad;  // pooled rows per event
     static constexpr int64_t ROWS_O = SEQ ? (int64_t)kSlices * SEQU + kPad : 2 * L_ + 2 * kPad;  // ConvT rows per event
+    // the ConvT output of the last level (u1) is stored in the quad layout that dec1 reads
+    static constexpr bool OUTQ = EPI == EPI_UP && (SEQ ? SEQ == kIvLen / 2 + kPad : L == kBins / 2);
+    static constexpr int RQ_O = quad_rows((int)ROWS_O - 2 * kPad);
     static constexpr bool DYN = DYN_;                       // tiles from the global counter
-    // output rows per tile: row 127 of a paired tile lacks O[128]; the fused final conv
-    // also needs two rows on each side
+    // output rows per tile: row 127 of a paired tile lacks O[128]
     static constexpr int ROWS_OK = PAIRED ? kTileM - 1 : kTileM;
-    static constexpr int STRIDE = EPI == EPI_FINAL ? ROWS_OK - 2 * kPad : ROWS_OK;
+    static constexpr int STRIDE = ROWS_OK;
     static constexpr int TPE = (L + STRIDE - 1) / STRIDE;    // tiles per event
     static constexpr int A_STAGE = align_up(PIN * ROWS * 16, 128);
     static constexpr int W_BYTES = TAPS * PIN * COUT * 16;
@@ -146,17 +148,15 @@ struct Cfg {
     static constexpr int UP_OFF = 0;
     static constexpr int A2_COL0 = NB * COLS_BUF;            // A2 buffers after the accumulators
     static constexpr int TMEM_COLS = pow2ceil(NB * COLS_BUF + 2 * A2_COLS);
-    // float parameters kept in shared memory: bias, bias2, column scales, final conv
-    static constexpr int NPAR = 2 * (COUT + N2) + (EPI == EPI_FINAL ? 5 * COUT + 1 : 0);
+    // float parameters kept in shared memory: bias, bias2, column scales
+    static constexpr int NPAR = 2 * (COUT + N2);
     static constexpr int OFF_W = 0;
     static constexpr int OFF_W2 = align_up(OFF_W + W_BYTES, 128);
     static constexpr int OFF_PAR = align_up(OFF_W2 + W2_BYTES, 128);
     static constexpr int OFF_A = align_up(OFF_PAR + 4 * NPAR, 128);
     static constexpr int OFF_A2 = OFF_A + STAGES * A_STAGE;
-    static constexpr int OFF_G = align_up(OFF_A2 + 2 * A2_BYTES, 128);
-    static constexpr int G_BYTES = EPI == EPI_FINAL ? 2 * 5 * kTileM * 4 : 0;
     // paired: each lane quarter's first O row, for the quarter above (two buffers)
-    static constexpr int OFF_X = align_up(OFF_G + G_BYTES, 128);
+    static constexpr int OFF_X = align_up(OFF_A2 + 2 * A2_BYTES, 128);
     static constexpr int X_BYTES = PAIRED ? 2 * 4 * COUT * 4 : 0;
     static constexpr int OFF_BAR = align_up(OFF_X + X_BYTES, 128);
     static constexpr int SMEM = OFF_BAR + 512;
@@ -168,8 +168,6 @@ struct Cfg {
     static_assert(N2 % 16 == 0 && N2 <= 256, "MMA N of the fused GEMM");
     static_assert(PIN % 2 == 0 || PAIR, "K planes come in pairs");
     static_assert(EPI != EPI_UP || P2 % 2 == 0, "fused GEMM K planes come in pairs");
-    static_assert(EPI != EPI_FINAL || ((COUT == kC0 || COUT == kC0Max) && (!PAIRED || COUT == kC0)),
-                  "final conv reads c0 channels");
     static_assert(TMEM_COLS <= 512, "TMEM columns");
     static_assert(OFF_PAR % 16 == 0 && COUT % 4 == 0 && N2 % 4 == 0, "parameters read as float4");
     static_assert(OFF_X % 16 == 0, "paired exchange in float4");
@@ -188,7 +186,7 @@ struct Cfg {
                            (EPI != EPI_POOL || (SEQ % 2 == 0 && LSEQ % 2 == 0))),
                   "per-interval geometry");
     static_assert(EPI != EPI_UP || CUP % 16 == 0, "16-column epilogue chunks");
-    static_assert(EWG == 1 || (EWG == 2 && EPI != EPI_FINAL && EPI_COLS % 16 == 0) ||
+    static_assert(EWG == 1 || (EWG == 2 && EPI_COLS % 16 == 0) ||
                   (EWG == 4 && EPI == EPI_UP && (COUT / 2) % 16 == 0 && (N2 / 2) % 16 == 0),
                   "epilogue warpgroups");
     static_assert(EPI != EPI_UP || N2 % 16 == 0, "ConvT columns in 16-column chunks");
@@ -197,11 +195,11 @@ struct Cfg {
 struct TcArgs {
     const unsigned char *inA, *inB;     // plane-major inputs (inB: skip half of the concat)
     unsigned char *out, *outp;          // conv or ConvT output; pooled output
-    float *logits;                      // EPI_FINAL: [n_events][L] float32
+    float *logits;                      // dec1: [n_events][4000] float32
     const unsigned char *w, *w2;        // packed weights (shared-memory image)
     const float *bias, *bias2;          // float32 biases
     const float *cs, *cs2;              // fp8: per-column dequantisation scales; 16-bit: null
-    const float *final_w;               // EPI_FINAL: W[t][ci] then b (float32)
+    const float *final_w;               // dec1: the final conv, W[t][ci] then b (float32)
     float out_inv, mid_inv;             // fp8: 1 / scale of the stored output and of A2
     float *amax;                        // calibration: running max |x| per scale slot, or null
     int amax_out, amax_mid;             // slots of the stored output and of A2 (kScale*)
@@ -215,13 +213,14 @@ struct TcArgs {
                                         // nothing arrives on, then the kernel unwinds
 };
 
-// Calibration: folds max |v| of 16 values (rows with valid = false count as 0) into the
+// Calibration: folds max |v| of N values (rows with valid = false count as 0) into the
 // warp maximum and lane 0 raises amax[slot] with an integer atomicMax on the float bits,
 // which orders non-negative floats correctly and does not depend on arrival order.
-__device__ __forceinline__ void amax_fold(float *amax, int slot, const float (&v)[16], bool valid) {
+template <int N>
+__device__ __forceinline__ void amax_fold(float *amax, int slot, const float (&v)[N], bool valid) {
     float m = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) m = fmaxf(m, fabsf(v[j]));
+    for (int j = 0; j < N; ++j) m = fmaxf(m, fabsf(v[j]));
     if (!valid) m = 0.0f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -230,14 +229,13 @@ __device__ __forceinline__ void amax_fold(float *amax, int slot, const float (&v
 
 // Barrier slots in shared memory (uint64 each). TFULL/TEMPTY/T2FULL follow the NB
 // accumulator buffers (tile i: buffer i % NB), so none of them can complete a second
-// phase before its waiters have seen the first; A2FULL/GREADY follow the two
-// shared-memory buffers of the fused ConvT operand and of the final conv's exchange
-// (tile i: i % 2).
+// phase before its waiters have seen the first; A2FULL follows the two
+// buffers of the fused ConvT operand (tile i: i % 2).
 constexpr int kRing = 12;    // tile-index ring: >= STAGES + NB tiles in flight
 template <class C> struct Bars {
     static constexpr int W = 0, FULL = 1, EMPTY = 1 + C::STAGES, TFULL = 1 + 2 * C::STAGES,
                          TEMPTY = TFULL + C::NB, T2FULL = TEMPTY + C::NB, A2FULL = T2FULL + C::NB,
-                         DRAIN = A2FULL + 2, GREADY = DRAIN + 1, XREADY = GREADY + 2,
+                         DRAIN = A2FULL + 2, XREADY = DRAIN + 1,
                          TIDF = XREADY + 2, TIDE = TIDF + kRing, N = TIDE + kRing;
     // after the barriers: TMEM address slot, abort flag, then the ring of tile indices
     static constexpr int RING_OFF = N * 8 + 16;
@@ -249,7 +247,7 @@ template <class C>
 __device__ __forceinline__ void tile_pos(int t, int &e, int &p0) {
     e = t / C::TPE;
     const int k = t % C::TPE;
-    p0 = C::EPI == EPI_FINAL ? k * C::STRIDE - kPad : k * C::STRIDE;
+    p0 = k * C::STRIDE;
 }
 
 // Per-interval layout: position p of the event lies in sequence s at position j of it;
@@ -498,6 +496,15 @@ __device__ __forceinline__ void lds16(const float *p, float (&v)[16]) {
     }
 }
 
+__device__ __forceinline__ void lds8(const float *p, float (&v)[8]) {
+    const float4 *q = reinterpret_cast<const float4 *>(p);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float4 x = q[i];
+        v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+    }
+}
+
 // Paired taps: conv columns [c0, c0 + W) of row m = E[m] + O[m + 1]. The O columns are
 // loaded first: lane 0 of each quarter publishes its O row into sx and arrives on xready
 // (`use`: how many times this barrier completed before, for its parity); O[m + 1] then
@@ -681,6 +688,14 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
     // output rows 2 j + r of sequence s (whole events: 2 p + r)
     const int64_t orow0 = C::SEQ ? (int64_t)sq * C::SEQU + 2 * jq + kPad : 2 * p + kPad;
     constexpr int PUP = C::CUP / C::PW;
+    // byte offset of storage row `row` of channel plane k, and of the next channel plane
+    auto at = [&](int k, int64_t row) {
+        return C::OUTQ ? quad_off(e, k, PUP, C::RQ_O, (int)row - kPad) : planar_off(e, k, PUP, ROWS_O, row);
+    };
+    constexpr size_t next_plane = C::OUTQ ? (size_t)4 * C::RQ_O * 16 : (size_t)ROWS_O * 16;
+    auto zero_row = [&](int64_t row) {
+        for (int k = 0; k < PUP; ++k) *reinterpret_cast<uint4 *>(a.out + at(k, row)) = make_uint4(0, 0, 0, 0);
+    };
 #pragma unroll 1
     for (int cc = 0; cc < NC; cc += LDW) {
         float vv[LDW];
@@ -706,27 +721,26 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
             }
             if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid && inseq);
             if (valid && inseq)
-                put16<C::PREC>(a.out + planar_off(e, co0 / C::PW, PUP, ROWS_O, orow0 + r),
-                          (size_t)ROWS_O * 16, v, a.out_inv);
+                put16<C::PREC>(a.out + at(co0 / C::PW, orow0 + r), next_plane, v, a.out_inv);
         }
     }
     if constexpr (C::SEQ != 0) {     // each output sequence's zero rows
         if (pads && valid && jq == 0) {
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, (int64_t)sq * C::SEQU);
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, (int64_t)sq * C::SEQU + 1);
+            zero_row((int64_t)sq * C::SEQU);
+            zero_row((int64_t)sq * C::SEQU + 1);
         }
         if (pads && valid && jq == C::LSEQ - 1 && sq == kSlices - 1) {   // the event's last two rows
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, (int64_t)kSlices * C::SEQU);
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, (int64_t)kSlices * C::SEQU + 1);
+            zero_row((int64_t)kSlices * C::SEQU);
+            zero_row((int64_t)kSlices * C::SEQU + 1);
         }
     } else {
         if (pads && p == 0) {
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, 0);
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, 1);
+            zero_row(0);
+            zero_row(1);
         }
         if (pads && p == C::L - 1) {
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, LO + kPad);
-            zero_planes(a.out, e, 0, PUP, PUP, ROWS_O, LO + kPad + 1);
+            zero_row(LO + kPad);
+            zero_row(LO + kPad + 1);
         }
     }
 }
@@ -736,11 +750,11 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
                          volatile int *ring, volatile int *abort, int warp, int lane) {
     using B = Bars<C>;
     uint64_t *tfull = bar + B::TFULL, *tempty = bar + B::TEMPTY, *a2full = bar + B::A2FULL,
-             *t2full = bar + B::T2FULL, *gready = bar + B::GREADY, *xready = bar + B::XREADY,
+             *t2full = bar + B::T2FULL, *xready = bar + B::XREADY,
              *tidf = bar + B::TIDF, *tide = bar + B::TIDE;
     const float *par = reinterpret_cast<const float *>(smem + C::OFF_PAR);
     const float *sbias = par, *sbias2 = par + C::COUT, *scs = par + C::COUT + C::N2,
-                *scs2 = scs + C::COUT, *sfin = par + 2 * (C::COUT + C::N2);
+                *scs2 = scs + C::COUT;
     const int q = warp & 3;                         // TMEM lane quarter of this warp
     const int m = q * 32 + lane;                    // tile row
     const int wg = (warp - 2) >> 2;                 // epilogue warpgroup
@@ -806,71 +820,6 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             mbar_arrive(&tempty[b]);
             continue;
         }
-        if constexpr (C::EPI == EPI_FINAL) {
-            constexpr int NCH = C::COUT / 16;       // 16-channel chunks of d1
-            float v[NCH][16];
-            if constexpr (C::PAIRED) {
-                if (!paired_cols<C, 16, false>(dcol, 0, sx, q, lane, &xready[ab], (uint32_t)(i >> 1), abort, v[0]))
-                    return false;
-            } else {
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch) tmem_ld16(dcol + 16 * ch, v[ch]);
-            }
-            tc_fence_before();
-            mbar_arrive(&tempty[b]);
-            float g[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                float bj[16], sc[16];
-                lds16(sbias + 16 * ch, bj);
-                if constexpr (!is16(C::PREC)) lds16(scs + 16 * ch, sc);
-                if constexpr (is16(C::PREC)) bias_leaky(v[ch], bj);
-                else scale_bias_leaky(v[ch], sc, bj);
-                if (!(valid && inseq)) {   // zero padding outside the event or its sequence
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[ch][j] = 0.0f;
-                }
-                if constexpr (CAL) amax_fold(a.amax, a.amax_out, v[ch], valid && inseq);
-                // the final conv's partial sums over this chunk's channels, in channel order:
-                // taps (0, 1) and (2, 3) as packed two-lane FMAs (each lane an fmaf), from
-                // weights stored per channel as (w0, w1, w2, w3), then tap 4
-                float2 g01 = make_float2(g[0], g[1]), g23 = make_float2(g[2], g[3]);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const float4 w4 = reinterpret_cast<const float4 *>(sfin)[16 * ch + j];
-                    const float2 vv = make_float2(v[ch][j], v[ch][j]);
-                    g01 = __ffma2_rn(make_float2(w4.x, w4.y), vv, g01);
-                    g23 = __ffma2_rn(make_float2(w4.z, w4.w), vv, g23);
-                }
-                g[0] = g01.x; g[1] = g01.y; g[2] = g23.x; g[3] = g23.y;
-                {
-                    float wf[16];
-                    lds16(sfin + 4 * C::COUT + 16 * ch, wf);
-                    float acc = g[4];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) acc = fmaf(wf[j], v[ch][j], acc);
-                    g[4] = acc;
-                }
-            }
-            float *sg = reinterpret_cast<float *>(smem + C::OFF_G) + ab * 5 * kTileM;
-#pragma unroll
-            for (int tp = 0; tp < 5; ++tp) sg[tp * kTileM + m] = g[tp];
-            // neighbours' partial sums: a bounded mbarrier among the 128 epilogue threads
-            mbar_arrive(&gready[ab]);
-            if (!mbar_wait(&gready[ab], ph_a, abort)) return false;
-            // per-interval layout: the logits of an interval's bins are its sequence's
-            // central positions [kIvPad, kIvPad + kSliceBins)
-            const bool out = !C::SEQ || (jq >= kIvPad && jq < kIvPad + kSliceBins);
-            if (m >= kPad && m < kPad + C::STRIDE && valid && out) {
-                // f(p) = b + sum_t g_t(p + t - 2), in tap order
-                float f = sfin[5 * C::COUT];
-#pragma unroll
-                for (int tp = 0; tp < 5; ++tp) f += sg[tp * kTileM + m + tp - 2];
-                if constexpr (C::SEQ != 0) a.logits[(size_t)e * kBins + sq * kSliceBins + jq - kIvPad] = f;
-                else a.logits[(size_t)e * C::L + p] = f;
-            }
-            continue;
-        }
         if constexpr (C::EPI == EPI_UP) {   // one warpgroup: conv, then the ConvT
             if (!epi_conv<C, C::COUT, CAL>(a, smem, sbias, scs, dcol, 0, ab, e, p, m, valid, sx,
                                       a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
@@ -932,11 +881,7 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
         if (k < C::COUT) v = C::EPI == EPI_CONVT ? a.bias[k % C::CUP] : a.bias[part * C::COUT + k];
         else if (k < C::COUT + C::N2) v = a.bias2[(k - C::COUT) % (C::CUP > 0 ? C::CUP : 1)];
         else if (k < 2 * C::COUT + C::N2) v = a.cs ? a.cs[part * C::COUT + k - C::COUT - C::N2] : 1.0f;
-        else if (k < 2 * (C::COUT + C::N2)) v = a.cs2 ? a.cs2[k - 2 * C::COUT - C::N2] : 1.0f;
-        else {   // the final conv: (w0, w1, w2, w3) per channel, then w4 per channel, then b
-            const int f = k - 2 * (C::COUT + C::N2);
-            v = f < 4 * C::COUT ? a.final_w[(f & 3) * C::COUT + (f >> 2)] : a.final_w[f];
-        }
+        else v = a.cs2 ? a.cs2[k - 2 * C::COUT - C::N2] : 1.0f;
         par[k] = v;
     }
     if (threadIdx.x == 0) {
@@ -952,8 +897,6 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
         }
         for (int b = 0; b < 2; ++b) mbar_init(&bar[B::A2FULL + b], 128 * ((C::EWG + 1) / 2));
         mbar_init(&bar[B::DRAIN], 1);
-        mbar_init(&bar[B::GREADY], 128);
-        mbar_init(&bar[B::GREADY + 1], 128);
         mbar_init(&bar[B::XREADY], 128 * ((C::EWG + 1) / 2));     // the conv epilogue's warpgroups
         mbar_init(&bar[B::XREADY + 1], 128 * ((C::EWG + 1) / 2));
         for (int r = 0; r < kRing; ++r) {
@@ -1051,9 +994,11 @@ cudaError_t launch_conv(const TcArgs &a, cudaStream_t s, const ProfHook *prof, c
 
 // Conv layers (0..5: enc2, enc3, enc4, dec3, dec2, dec1) whose taps are stacked in pairs
 // along N: where it measured faster, the 16-bit dec3 (44 -> 28 MMAs per tile) and dec2. The
-// FP8 form already halves the MMAs (K = 32) and measured slower paired; dec1 is bound by
-// its epilogue.
+// FP8 form already halves the MMAs (K = 32) and measured slower paired; dec1 has a kernel of
+// its own.
 constexpr bool conv_paired(int li, int prec) { return (li == 3 || li == 4) && is16(prec); }
+
+#include "dec1_tc.cuh"
 
 template <int PREC> struct Net {
     static constexpr bool FUSED_ENC = true;    // enc2, enc3 and enc4 + up3 run as k_enc_tc
@@ -1067,7 +1012,7 @@ template <int PREC> struct Net {
                         true>;                                                         // 1 CTA/SM
     using Dec2Up1 = Cfg<PREC, 32, 32, 32, 2000, EPI_UP, 16, 3, 2, 96, 3, conv_paired(4, PREC), false,
                         true>;                                                         // 2
-    using Dec1Final = Cfg<PREC, 16, 16, 16, 4000, EPI_FINAL, 0, 3, 1, 64, 4, conv_paired(5, PREC)>; // 5
+    using Last = Dec1<PREC, 16, 4000>;                                                  // 2
 };
 
 // The per-interval layout (§3's batch of 40 intervals, each its own sequence of kIvLen =
@@ -1085,8 +1030,7 @@ template <int PREC> struct NetIv {
                         false, true, S3>;
     using Dec3Up2 = Cfg<PREC, 64, 64, 64, L2, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false, true, S2>;
     using Dec2Up1 = Cfg<PREC, 32, 32, 32, L1, EPI_UP, 16, 3, 2, 128, 3, conv_paired(4, PREC), false, true, S1>;
-    using Dec1Final = Cfg<PREC, 16, 16, 16, L0, EPI_FINAL, 0, 3, 1, 64, 4, conv_paired(5, PREC), false, false,
-                          S0>;
+    using Last = Dec1<PREC, 16, L0, S0>;
 };
 
 #include "enc_tc.cuh"
@@ -1107,7 +1051,7 @@ template <int PREC> struct Net32 {
                      false, false, 0, SP>;
     using Up2 = Cfg<PREC, 128, 0, 128, 1000, EPI_CONVT, 64, 3, 2, 128, 2>;
     using Dec2Up1 = Cfg<PREC, 64, 64, 64, 2000, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false, true>;
-    using Dec1Final = Cfg<PREC, 32, 32, 32, 4000, EPI_FINAL, 0, 3, 1, 96, 4>;
+    using Last = Dec1<PREC, 32, 4000>;
 };
 
 // Index of each tensor-core layer in TcNet::w: enc2, enc3, enc4, dec3, dec2, dec1, up3, up2, up1
@@ -1199,8 +1143,11 @@ bool tc_pack_weights(int precision, const std::vector<LayerF32> &layers, const f
                             // part tap-major planes of cout / sp rows (enc4, and dec3 in e4m3)
                             // or the paired groups (16-bit dec3)
                             const int cl = cout / sp, cp = co % cl;
+                            // dec1: each plane holds its taps in descending order (windows of it are
+                            // the stacked MMAs' operands)
                             const size_t row =
-                                wide && li == 3 && is16(precision)
+                                li == 5 ? ((size_t)k * 5 + (4 - t)) * cout + co
+                                : wide && li == 3 && is16(precision)
                                     ? (size_t)(co / cl) * 5 * pin * cl + (size_t)(t / 2) * pin * 2 * cl +
                                           (size_t)k * (t < 4 ? 2 * cl : cl) + (t % 2) * cl + cp
                                 : wide && (li == 2 || li == 3)
@@ -1340,7 +1287,7 @@ static cudaError_t run_tc(const TcNet &n, const UnetBuffers &b, int ne, const in
     a.inA = U(b.up); a.inB = U(b.e1); a.out = nullptr; a.w2 = nullptr; a.bias2 = nullptr; a.sched = sched(5);
     a.cs2 = nullptr; a.logits = b.logits; a.final_w = n.final_w; a.amax_out = kScaleD1;
     a.w = W(5); a.bias = n.b[5]; a.cs = cs(5);
-    return launch_conv<typename N::Dec1Final>(a, s, prof, "dec1_final", n.ctas_per_sm[5]);
+    return launch_dec1<typename N::Last>(a, s, prof, n.ctas_per_sm[5]);
 }
 
 // The wide network (base width 32). Activation slots by liveness: e1 | e2 | e3 | deep = e4,
@@ -1397,7 +1344,7 @@ static cudaError_t run_tc32(const TcNet &n, const UnetBuffers &b, int ne, const 
     a.inA = U(b.deep); a.inB = U(b.e1); a.out = nullptr; a.w2 = nullptr; a.bias2 = nullptr; a.sched = sched(5);
     a.cs2 = nullptr; a.logits = b.logits; a.final_w = n.final_w; a.amax_out = kScaleD1;
     a.w = W(5); a.bias = n.b[5]; a.cs = cs(5);
-    return launch_conv<typename N::Dec1Final>(a, s, prof, "dec1_final", n.ctas_per_sm[5]);
+    return launch_dec1<typename N::Last>(a, s, prof, n.ctas_per_sm[5]);
 }
 
 // The encoder kernel alone with its enc2 MMA warp stalled for stall_us (tests of the bounded waits).

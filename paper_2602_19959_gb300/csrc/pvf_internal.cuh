@@ -206,6 +206,15 @@ __host__ __device__ __forceinline__ size_t planar_off(int64_t e, int k, int plan
     return ((size_t)(e * planes + k) * (size_t)rows_e + (size_t)row) * 16;
 }
 
+// Quad layout of the last level's inputs in the tensor-core forms (e1 and u1): each channel
+// plane is split by the position's residue modulo 4, so that four consecutive positions lie at
+// the same row of four planes. Position p (-2 .. L + 1, the pads included) of channel plane k:
+// plane 4 k + (p & 3), row (p >> 2) + 1 of quad_rows(L).
+__host__ __device__ constexpr int quad_rows(int L) { return (L + 1) / 4 + 2; }
+__host__ __device__ __forceinline__ size_t quad_off(int64_t e, int k, int planes, int rows, int p) {
+    return ((size_t)((e * planes + k) * 4 + (p & 3)) * (size_t)rows + (size_t)((p >> 2) + 1)) * 16;
+}
+
 // e4m3 codes of v[0..N) * inv_scale packed four to a word (v[4 i] in the low byte of
 // out[i]), two per conversion instruction (round to nearest even, saturating to the
 // largest finite value, as __nv_fp8_e4m3(float)).
@@ -241,7 +250,8 @@ struct FrontArgs {
     const float *enc1;           // kEnc1Floats
     const float *hist_in;        // non-null: skip steps 1-2, read histograms (global rows)
     float *hist_out;             // nullable, global rows [ev_base + e]
-    void *e1;                    // chunk-local padded [n][4004][16]; null: steps 1-2 only
+    void *e1;                    // chunk-local padded [n][4004][16] (tensor-core forms: the quad
+                                 // layout); null: steps 1-2 only
     void *p1;                    // chunk-local padded [n][2004][16]
     float e1_inv_scale;          // fp8 only: 1 / scale of e1/p1
     float *amax;                 // calibration: max |e1| into amax[0], or null
