@@ -88,7 +88,7 @@ typedef struct {
                                       dec2_up1, dec1_final. The first three have no effect for
                                       whole events at width 16, where one kernel with one CTA
                                       per SM runs these layers                                */
-    int32_t tail_ctas_per_sm;      /* peak finder: 1..8                                         */
+    int32_t tail_ctas_per_sm;      /* peak finder: 1..4 (float32 form: 1..2)                     */
 } pvf_schedule;
 
 /* Creation-time plan (§3: TensorSpec freezing batch dimensions, channels, length and

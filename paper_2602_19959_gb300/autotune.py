@@ -28,7 +28,7 @@ FAMILIES = ("front", "enc2", "enc3", "enc4_up3", "dec3_up2", "dec2_up1", "dec1_f
 # CTAs per SM tried for each family (0 = as many as fit; the library clamps larger values)
 GRID_CANDIDATES = {"front": (1, 2, 3, 4), "enc2": (2, 3, 4, 6), "enc3": (1, 2, 3, 4), "enc4_up3": (1,),
                    "dec3_up2": (1,), "dec2_up1": (1, 2), "dec1_final": (2, 3, 4, 5),
-                   "tail": (1, 2, 4, 8)}
+                   "tail": (1, 2, 4)}
 TUNED_DIR = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned")
 
 

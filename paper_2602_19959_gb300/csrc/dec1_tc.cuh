@@ -274,7 +274,13 @@ __device__ bool dec1_epilogue(const TcArgs &a, unsigned char *smem, uint64_t *ba
                 if (((in >> j) & 1u) && jq[j] >= kIvPad && jq[j] < kIvPad + kSliceBins)
                     a.logits[(size_t)e * kBins + sq[j] * kSliceBins + jq[j] - kIvPad] = f[j];
         } else {
-            *reinterpret_cast<float4 *>(a.logits + (size_t)e * C::L + p0) = make_float4(f[0], f[1], f[2], f[3]);
+            float *out = a.logits + (size_t)e * C::L + p0;
+            if ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0) {
+                *reinterpret_cast<float4 *>(out) = make_float4(f[0], f[1], f[2], f[3]);
+            } else {                                // a caller's buffer, aligned to 4 bytes only
+#pragma unroll
+                for (int j = 0; j < 4; ++j) out[j] = f[j];
+            }
         }
     }
     return true;

@@ -502,6 +502,11 @@ static cudaError_t run_chunk(pvf_handle *h, const pvf_tracks_soa *tracks, const 
     int32_t *flags = reinterpret_cast<int32_t *>(h->pool + h->plan.ev_flag);
     int32_t *n_copy = n_dyn ? reinterpret_cast<int32_t *>(h->pool + h->plan.status + kDynCountOff) : nullptr;
     const int prec = h->cfg.precision;
+    // tensor-core forms: the logits a caller asked for are written by dec1, in place of the
+    // pool's (the peak finder then reads them there)
+    UnetBuffers buf = h->buf;
+    const bool direct = logit_out && prec != PVF_FP32;
+    if (direct) buf.logits = logit_out + (size_t)ev_base * kBins;
     cudaError_t err = cudaSuccess;
     const ProfHook *prof = h->prof.on ? &h->hook : nullptr;
     if (run_front) {
@@ -544,10 +549,10 @@ static cudaError_t run_chunk(pvf_handle *h, const pvf_tracks_soa *tracks, const 
     }
     if (run_unet) {
         if (prec == PVF_FP32) err = launch_unet_f32(h->cw, h->buf, n, h->cfg.per_interval != 0, s, prof);
-        else err = launch_unet_tc(h->tc, h->buf, n, n_copy, ev_base, s, prof);
+        else err = launch_unet_tc(h->tc, buf, n, n_copy, ev_base, s, prof);
         if (err != cudaSuccess) return err;
     }
-    if (run_tail) {
+    if (run_tail && (pv_count || prec == PVF_FP32)) {     // logits alone: dec1 has written them
         ProfScope ps(prof, "tail", s);
         TailArgs t{};
         t.d1 = h->buf.deep;
@@ -556,7 +561,7 @@ static cudaError_t run_chunk(pvf_handle *h, const pvf_tracks_soa *tracks, const 
         t.ev_flag = logit_in ? nullptr : flags;
         if (!logit_in && prec != PVF_FP32) {
             // tensor-core forms: the final conv ran in dec1's epilogue; peaks only
-            t.logit_in = h->buf.logits;
+            t.logit_in = buf.logits;
             t.logit_in_base = ev_base;
         }
         t.d1_scale = h->act_scale[kScaleD1];
@@ -565,7 +570,7 @@ static cudaError_t run_chunk(pvf_handle *h, const pvf_tracks_soa *tracks, const 
         t.iv = h->cfg.per_interval;
         t.n_events = n;
         t.ev_base = ev_base;
-        t.logit_out = logit_out;
+        t.logit_out = direct ? nullptr : logit_out;
         t.pv_z = pv_z;
         t.pv_count = pv_count;
         t.max_pv = h->cfg.max_pv_per_event;
