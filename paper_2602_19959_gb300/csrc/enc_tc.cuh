@@ -44,16 +44,15 @@ template <class N> struct Enc {
     static constexpr int COL2 = 0, COL3 = COL2 + 2 * C2::COUT, COL4 = COL3 + 2 * C3::COUT,
                          COL5 = COL4 + C4::COUT, COLA = COL5 + C4::N2, TMEM_COLS = 512;
     static_assert(COLA + C4::A2_COLS <= TMEM_COLS, "TMEM columns");
-    // shared memory: weights, parameters, p1 stages, p2 and p3 tiles, barriers
+    // shared memory: weights, p1 stages, p2 and p3 tiles, barriers
     static constexpr int OFF_W2 = 0, OFF_W3 = align_up(OFF_W2 + C2::W_BYTES, 128),
                          OFF_W4 = align_up(OFF_W3 + C3::W_BYTES, 128),
                          OFF_W5 = align_up(OFF_W4 + C4::W_BYTES, 128),
-                         OFF_PAR = align_up(OFF_W5 + C4::W2_BYTES, 128);
-    // parameters (floats): bias then column scales of enc2, enc3, enc4, up3
+                         OFF_A = align_up(OFF_W5 + C4::W2_BYTES, 128);
+    // launch parameters (floats): biases of enc2, enc3, enc4, up3, then (e4m3) their column scales
     static constexpr int PB2 = 0, PB3 = PB2 + C2::COUT, PB4 = PB3 + C3::COUT, PB5 = PB4 + C4::COUT,
                          PS2 = PB5 + C4::CUP, PS3 = PS2 + C2::COUT, PS4 = PS3 + C3::COUT, PS5 = PS4 + C4::COUT,
-                         NPAR = PS5 + C4::N2;
-    static constexpr int OFF_A = align_up(OFF_PAR + 4 * NPAR, 128);
+                         NPAR = is16(C2::PREC) ? PS2 : PS5 + C4::N2;
     static constexpr int OFF_P2 = OFF_A + ST * C2::A_STAGE;
     static constexpr int OFF_P3 = OFF_P2 + NP2 * P2_BYTES;
     static constexpr int OFF_BAR = OFF_P3 + NP3 * P3_BYTES;
@@ -250,7 +249,7 @@ struct EncPool {
     unsigned char *out;                       // stored tensor, at this thread's row of an event's first tile
     size_t ev_bytes;                          // bytes per event of it
     uint32_t plane;                           // bytes per plane of it
-    uint32_t bias, scale;
+    int bias, scale;                          // places in the parameter block
     float out_inv;
     int cols, len;                            // channels, positions per event
     uint32_t bufs, buf_bytes;                 // operand tiles of the next layer
@@ -265,8 +264,8 @@ struct EncPool {
 // zero rows before it. The even lane of a row pair writes the first 8 of each 16 channels (a
 // plane in 16 bits, half a plane's row in e4m3), the odd lane the last 8. The accumulator is
 // released (L.free) as soon as its last columns are in registers.
-template <int PREC, bool CAL, int PLANE>
-__device__ __forceinline__ void enc_epi(const EncPool &L, const TcArgs &a, unsigned char *dst, bool odd, bool valid, bool st,
+template <int PREC, bool CAL, int PLANE, class P>
+__device__ __forceinline__ void enc_epi(const EncPool &L, const P &par, const TcArgs &a, unsigned char *dst, bool odd, bool valid, bool st,
                                         uint32_t buf, int row, uint32_t nbuf, int nrow, int lead) {
     const uint32_t half = !odd ? 0 : is16(PREC) ? PLANE : 8;
     const bool edge = nbuf || lead >= 0;
@@ -280,12 +279,12 @@ __device__ __forceinline__ void enc_epi(const EncPool &L, const TcArgs &a, unsig
             tc_fence_before();
             mbar_arrive_at(L.free);
         }
-        lds16_at(L.bias + 4 * c0, bj);
+        ldp(par, L.bias + c0, bj);
         if constexpr (is16(PREC)) {
             bias_leaky(v, bj);
         } else {
             float sc[16];
-            lds16_at(L.scale + 4 * c0, sc);
+            ldp(par, L.scale + c0, sc);
             scale_bias_leaky(v, sc, bj);
         }
         if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid);
@@ -335,7 +334,7 @@ __device__ __forceinline__ void enc_epi(const EncPool &L, const TcArgs &a, unsig
 // tiles [s0, s1) are stored. This loop's scalar work is a sixth of the kernel's instructions, so
 // nothing in it is recomputed per tile that a unit or the thread fixes.
 template <class E, bool CAL>
-__device__ bool enc_pool_role(const EncPool &L, const TcArgs &a, int half, int m, int nu, int lg, volatile int *abort) {
+__device__ bool enc_pool_role(const EncPool &L, const ParBlock<E::NPAR> &par, const TcArgs &a, int half, int m, int nu, int lg, volatile int *abort) {
     constexpr int PREC = E::C2::PREC;
     static_assert(E::NP2 == 3 && E::NP3 == 3 && E::RING == 8 && E::C3::ROWS == E::C4::ROWS, "operand tiles");
     const bool odd = (m & 1) != 0;
@@ -372,7 +371,7 @@ __device__ bool enc_pool_role(const EncPool &L, const TcArgs &a, int half, int m
                 nbuf = L.bufs + (up ? (slot == 2 ? 0 : slot + 1) : (slot == 0 ? 2 : slot - 1)) * L.buf_bytes;
                 nrow = up ? row - kTileM : row + kTileM;
             }
-            enc_epi<PREC, CAL, E::C3::ROWS * 16>(L, a, out + (size_t)i * (kTileM * 16), odd, valid, st, buf, row, nbuf, nrow,
+            enc_epi<PREC, CAL, E::C3::ROWS * 16>(L, par, a, out + (size_t)i * (kTileM * 16), odd, valid, st, buf, row, nbuf, nrow,
                                                  i == 0 && m < 4 ? m >> 1 : -1);
             fence_proxy_async_smem();     // the operand rows -> visible to the tensor core
             mbar_arrive_at(L.done + 8 * ((n0 + i - ta) & 7));
@@ -391,7 +390,7 @@ __device__ bool enc_pool_role(const EncPool &L, const TcArgs &a, int half, int m
 }
 
 template <class E, bool CAL>
-__global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant__ EncArgs g) {
+__global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant__ EncArgs g, const __grid_constant__ ParBlock<E::NPAR> par) {
     using C2 = typename E::C2;
     using C3 = typename E::C3;
     using C4 = typename E::C4;
@@ -400,19 +399,6 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + E::NBAR);
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *par = reinterpret_cast<float *>(smem + E::OFF_PAR);
-    for (int q = threadIdx.x; q < E::NPAR; q += E::THREADS) {
-        float v;
-        if (q < E::PB3) v = g.c2.bias[q - E::PB2];
-        else if (q < E::PB4) v = g.c3.bias[q - E::PB3];
-        else if (q < E::PB5) v = g.c4.bias[q - E::PB4];
-        else if (q < E::PS2) v = g.c4.bias2[q - E::PB5];
-        else if (q < E::PS3) v = g.c2.cs ? g.c2.cs[q - E::PS2] : 1.0f;
-        else if (q < E::PS4) v = g.c3.cs ? g.c3.cs[q - E::PS3] : 1.0f;
-        else if (q < E::PS5) v = g.c4.cs ? g.c4.cs[q - E::PS4] : 1.0f;
-        else v = g.c4.cs2 ? g.c4.cs2[q - E::PS5] : 1.0f;
-        par[q] = v;
-    }
     if (threadIdx.x == 0) {
         for (int b = 0; b < E::NBAR; ++b) {
             // epilogue-to-MMA barriers count a warpgroup's threads, the others one arrival
@@ -471,8 +457,8 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
                 L.plane = (two ? C2::ROWS_E : C3::ROWS_E) * 16;
                 L.ev_bytes = (size_t)L.plane * (two ? C2::POUT : C3::POUT);
                 L.out = a.out + (m + kPad) * 16;
-                L.bias = smem_u32(par + (two ? E::PB2 : E::PB3));
-                L.scale = smem_u32(par + (two ? E::PS2 : E::PS3));
+                L.bias = two ? E::PB2 : E::PB3;
+                L.scale = two ? E::PS2 : E::PS3;
                 L.out_inv = a.out_inv;
                 L.cols = two ? C2::COUT : C3::COUT;
                 L.len = two ? C2::L : C3::L;
@@ -484,9 +470,8 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
                 L.done = smem_u32(bar + (two ? E::D2 : E::D3));
                 L.acc = lt + (two ? E::COL2 : E::COL3) + half * L.cols;
                 L.up = two ? 2 : 1;
-                ok = enc_pool_role<E, CAL>(L, a, half, m, nu, lg, abort);
+                ok = enc_pool_role<E, CAL>(L, par, a, half, m, nu, lg, abort);
             } else {
-                const float *sp = par;
                 int n4 = 0;
                 for (int u = blockIdx.x; ok && u < nu; u += gridDim.x) {
                     const EncUnit x = enc_unit<E>(u, lg);
@@ -497,7 +482,7 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
                             if (!mbar_wait(&bar[E::T4F], n4 & 1, abort) ||
                                 (n4 > 0 && !mbar_wait(&bar[E::A2E], (n4 - 1) & 1, abort))) { ok = false; break; }
                             tc_fence_after();
-                            epi_conv<C4, C4::COUT, CAL, 16>(g.c4, smem, sp + E::PB4, sp + E::PS4, lt + E::COL4, 0, 0, x.e, p, m,
+                            epi_conv<C4, C4::COUT, CAL, 16>(g.c4, smem, par, E::PB4, E::PS4, lt + E::COL4, 0, 0, x.e, p, m,
                                                    valid, nullptr, lt + E::COLA);
                             tmem_st_wait();
                             tc_fence_before();
@@ -506,7 +491,7 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
                         } else {           // ConvT accumulator -> u3
                             if (!mbar_wait(&bar[E::T5F], n4 & 1, abort)) { ok = false; break; }
                             tc_fence_after();
-                            epi_up<C4, C4::N2, CAL, 16>(g.c4, sp + E::PB5, sp + E::PS5, lt + E::COL5, 0, x.e, p, valid, true);
+                            epi_up<C4, C4::N2, CAL, 16>(g.c4, par, E::PB5, E::PS5, lt + E::COL5, 0, x.e, p, valid, true);
                             tc_fence_before();
                             mbar_arrive(&bar[E::T5E]);
                         }
@@ -539,5 +524,16 @@ cudaError_t launch_enc(const EncArgs &g, cudaStream_t s, const ProfHook *prof) {
     if (err != cudaSuccess) return err;
     const int grid = (int64_t)g.c2.n_events * E::T4N < sms ? g.c2.n_events * E::T4N : sms;
     ProfScope ps(prof, "enc_up3", s);
-    return launch_pdl(k_enc_tc<E, CAL>, dim3(grid), dim3(E::THREADS), (size_t)smem, s, g);
+    ParBlock<E::NPAR> par;
+    par.set(E::PB2, g.c2.bias, E::C2::COUT);
+    par.set(E::PB3, g.c3.bias, E::C3::COUT);
+    par.set(E::PB4, g.c4.bias, E::C4::COUT);
+    par.set(E::PB5, g.c4.bias2, E::C4::CUP);
+    if constexpr (!is16(E::C2::PREC)) {
+        par.set(E::PS2, g.c2.cs, E::C2::COUT);
+        par.set(E::PS3, g.c3.cs, E::C3::COUT);
+        par.set(E::PS4, g.c4.cs, E::C4::COUT);
+        par.set(E::PS5, g.c4.cs2, E::C4::N2);
+    }
+    return launch_pdl(k_enc_tc<E, CAL>, dim3(grid), dim3(E::THREADS), (size_t)smem, s, g, par);
 }

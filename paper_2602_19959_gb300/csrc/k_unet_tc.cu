@@ -148,12 +148,13 @@ struct Cfg {
     static constexpr int UP_OFF = 0;
     static constexpr int A2_COL0 = NB * COLS_BUF;            // A2 buffers after the accumulators
     static constexpr int TMEM_COLS = pow2ceil(NB * COLS_BUF + 2 * A2_COLS);
-    // float parameters kept in shared memory: bias, bias2, column scales
-    static constexpr int NPAR = 2 * (COUT + N2);
+    // launch parameters: bias (every part's), bias2, and for e4m3 their column scales
+    static constexpr int NBIAS = EPI == EPI_CONVT ? CUP : NSPLIT_ * COUT;
+    static constexpr int NSC = is16(PREC) ? 0 : NSPLIT_ * COUT, NSC2 = is16(PREC) ? 0 : N2;
+    static constexpr int QB = 0, QB2 = QB + NBIAS, QS = QB2 + (N2 ? CUP : 0), QS2 = QS + NSC, NPAR = QS2 + NSC2;
     static constexpr int OFF_W = 0;
     static constexpr int OFF_W2 = align_up(OFF_W + W_BYTES, 128);
-    static constexpr int OFF_PAR = align_up(OFF_W2 + W2_BYTES, 128);
-    static constexpr int OFF_A = align_up(OFF_PAR + 4 * NPAR, 128);
+    static constexpr int OFF_A = align_up(OFF_W2 + W2_BYTES, 128);
     static constexpr int OFF_A2 = OFF_A + STAGES * A_STAGE;
     // paired: each lane quarter's first O row, for the quarter above (two buffers)
     static constexpr int OFF_X = align_up(OFF_A2 + 2 * A2_BYTES, 128);
@@ -169,7 +170,7 @@ struct Cfg {
     static_assert(PIN % 2 == 0 || PAIR, "K planes come in pairs");
     static_assert(EPI != EPI_UP || P2 % 2 == 0, "fused GEMM K planes come in pairs");
     static_assert(TMEM_COLS <= 512, "TMEM columns");
-    static_assert(OFF_PAR % 16 == 0 && COUT % 4 == 0 && N2 % 4 == 0, "parameters read as float4");
+    static_assert(NBIAS % 4 == 0 && CUP % 4 == 0 && N2 % 4 == 0, "parameters read as float4");
     static_assert(OFF_X % 16 == 0, "paired exchange in float4");
     static_assert(STAGES >= 2 && STAGES <= 6, "stages");
     static_assert(NB >= 2 && NB <= 4, "accumulator buffers");
@@ -197,8 +198,8 @@ struct TcArgs {
     unsigned char *out, *outp;          // conv or ConvT output; pooled output
     float *logits;                      // dec1: [n_events][4000] float32
     const unsigned char *w, *w2;        // packed weights (shared-memory image)
-    const float *bias, *bias2;          // float32 biases
-    const float *cs, *cs2;              // fp8: per-column dequantisation scales; 16-bit: null
+    const float *bias, *bias2;          // float32 biases: host (dec1: device)
+    const float *cs, *cs2;              // fp8: per-column dequantisation scales, likewise; 16-bit: null
     const float *final_w;               // dec1: the final conv, W[t][ci] then b (float32)
     float out_inv, mid_inv;             // fp8: 1 / scale of the stored output and of A2
     float *amax;                        // calibration: running max |x| per scale slot, or null
@@ -212,6 +213,24 @@ struct TcArgs {
                                         // MMA thread first waits this long on a barrier that
                                         // nothing arrives on, then the kernel unwinds
 };
+
+// The biases (and e4m3 column scales) of a kernel's layer, passed as launch parameters: the
+// epilogues read them through the constant cache. In shared memory each 16-byte read of one
+// address by a whole warp still took four cycles of the port that feeds the MMAs their
+// operands: a third of the traffic there in the fused encoder, a fifth in dec3_up2.
+template <int N> struct ParBlock {
+    float4 v[(N + 3) / 4];
+    __host__ void set(int at, const float *src, int n, float fill = 1.0f) {
+        for (int i = 0; i < n; ++i) reinterpret_cast<float *>(v)[at + i] = src ? src[i] : fill;
+    }
+};
+template <int N, int M> __device__ __forceinline__ void ldp(const ParBlock<N> &p, int at, float (&x)[M]) {
+#pragma unroll
+    for (int i = 0; i < M / 4; ++i) {
+        const float4 q = p.v[at / 4 + i];
+        x[4 * i] = q.x; x[4 * i + 1] = q.y; x[4 * i + 2] = q.z; x[4 * i + 3] = q.w;
+    }
+}
 
 // Calibration: folds max |v| of N values (rows with valid = false count as 0) into the
 // warp maximum and lane 0 raises amax[slot] with an integer atomicMax on the float bits,
@@ -484,18 +503,7 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
     return ok;
 }
 
-// 16 consecutive parameters from shared memory in four 16-byte loads (p 16-byte aligned):
-// the epilogues read their biases, scales and final-conv weights per tile, and scalar
-// broadcast loads made the shared-memory pipe the bottleneck of the final conv.
-__device__ __forceinline__ void lds16(const float *p, float (&v)[16]) {
-    const float4 *q = reinterpret_cast<const float4 *>(p);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 x = q[i];
-        v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
-    }
-}
-
+// 8 consecutive parameters from shared memory in two 16-byte loads (p 16-byte aligned).
 __device__ __forceinline__ void lds8(const float *p, float (&v)[8]) {
     const float4 *q = reinterpret_cast<const float4 *>(p);
 #pragma unroll
@@ -565,9 +573,9 @@ __device__ __forceinline__ bool paired_cols(uint32_t dcol, int c0, float *sx, in
 // CAL: a calibration pass, which also records the largest stored magnitudes (its code, in every
 // 16-column block, stays out of the kernels that serve: they would not fit the instruction
 // cache as well).
-template <class C, int NC, bool CAL, int LDW = C::ldw(NC)>
-__device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, const float *sbias,
-                                         const float *scs, uint32_t dcol, int c_beg, int ab, int e,
+template <class C, int NC, bool CAL, int LDW = C::ldw(NC), class P>
+__device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, const P &par, int pbias, int pscale,
+                                         uint32_t dcol, int c_beg, int ab, int e,
                                          int p, int m, bool valid, float *sx = nullptr,
                                          uint32_t a2t = 0, bool inseq = true, uint64_t *xready = nullptr,
                                          uint32_t xuse0 = 0, volatile int *abort = nullptr) {
@@ -592,14 +600,14 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
         for (int h = 0; h < LDW / 16; ++h) {
             const int c0 = c_beg + cc + 16 * h;
             float v[16], bj[16];
-            lds16(sbias + c0, bj);
+            ldp(par, pbias + c0, bj);
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = vv[16 * h + j];
             if constexpr (is16(C::PREC)) {
                 bias_leaky(v, bj);
             } else {
                 float sc[16];
-                lds16(scs + c0, sc);
+                ldp(par, pscale + c0, sc);
                 scale_bias_leaky(v, sc, bj);
             }
             if constexpr (C::SEQ != 0) {
@@ -676,9 +684,8 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
 // Fused ConvT columns [n_beg, n_beg + NC) (n = r * CUP + co: output row 2p + r, channel
 // co): bias, LeakyReLU, store; the thread of p = 0 / L - 1 (with pads) zeroes the pads.
 // r0: the first output-row parity of these columns (the ConvT GEMM split by r: its part).
-template <class C, int NC, bool CAL, int LDW = NC % 32 == 0 ? 32 : 16>
-__device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, const float *scs2,
-                                       uint32_t dcol, int n_beg, int e, int p, bool valid, bool pads,
+template <class C, int NC, bool CAL, int LDW = NC % 32 == 0 ? 32 : 16, class P>
+__device__ __forceinline__ void epi_up(const TcArgs &a, const P &par, int pbias, int pscale, uint32_t dcol, int n_beg, int e, int p, bool valid, bool pads,
                                        int r0 = 0) {
     constexpr int LO = 2 * C::L;
     constexpr int64_t ROWS_O = C::ROWS_O;
@@ -709,14 +716,14 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
             const int c0 = n_beg + cc + 16 * h;
             const int r = r0 + c0 / C::CUP, co0 = c0 % C::CUP;
             float v[16], bj[16];
-            lds16(sbias2 + co0, bj);
+            ldp(par, pbias + co0, bj);
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = vv[16 * h + j];
             if constexpr (is16(C::PREC)) {
                 bias_leaky(v, bj);
             } else {
                 float sc[16];
-                lds16(scs2 + c0, sc);
+                ldp(par, pscale + c0, sc);
                 scale_bias_leaky(v, sc, bj);
             }
             if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid && inseq);
@@ -746,15 +753,12 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const float *sbias2, con
 }
 
 template <class C, bool CAL>
-__device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, uint32_t tmem,
+__device__ bool epilogue(const TcArgs &a, const ParBlock<C::NPAR> &par, unsigned char *smem, uint64_t *bar, uint32_t tmem,
                          volatile int *ring, volatile int *abort, int warp, int lane) {
     using B = Bars<C>;
     uint64_t *tfull = bar + B::TFULL, *tempty = bar + B::TEMPTY, *a2full = bar + B::A2FULL,
              *t2full = bar + B::T2FULL, *xready = bar + B::XREADY,
              *tidf = bar + B::TIDF, *tide = bar + B::TIDE;
-    const float *par = reinterpret_cast<const float *>(smem + C::OFF_PAR);
-    const float *sbias = par, *sbias2 = par + C::COUT, *scs = par + C::COUT + C::N2,
-                *scs2 = scs + C::COUT;
     const int q = warp & 3;                         // TMEM lane quarter of this warp
     const int m = q * 32 + lane;                    // tile row
     const int wg = (warp - 2) >> 2;                 // epilogue warpgroup
@@ -794,7 +798,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             if (wg < PER) {     // conv accumulator -> ConvT operand
                 if (!mbar_wait(&tfull[b], ph_b, abort)) return false;
                 tc_fence_after();
-                if (!epi_conv<C, C::COUT / PER, CAL>(a, smem, sbias, scs, dcol, part * (C::COUT / PER), ab, e, p, m,
+                if (!epi_conv<C, C::COUT / PER, CAL>(a, smem, par, C::QB, C::QS, dcol, part * (C::COUT / PER), ab, e, p, m,
                                                 valid, sx, a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
                                                 (uint32_t)(i >> 1) * C::xchunks(C::COUT / PER), abort))
                     return false;
@@ -805,7 +809,7 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             } else {            // ConvT accumulator -> output; frees the buffer
                 if (!mbar_wait(&t2full[b], ph_b, abort)) return false;
                 tc_fence_after();
-                epi_up<C, C::N2 / PER, CAL>(a, sbias2, scs2, dcol, part * (C::N2 / PER), e, p, valid, part == 0);
+                epi_up<C, C::N2 / PER, CAL>(a, par, C::QB2, C::QS2, dcol, part * (C::N2 / PER), e, p, valid, part == 0);
                 tc_fence_before();
                 mbar_arrive(&tempty[b]);
             }
@@ -814,14 +818,14 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
         if (!mbar_wait(&tfull[b], ph_b, abort)) return false;
         tc_fence_after();
         if constexpr (C::EPI == EPI_CONVT) {   // the ConvT GEMM: this warpgroup's columns
-            epi_up<C, C::EPI_COLS, CAL>(a, sbias, scs, dcol, wg * C::EPI_COLS, e, p, valid, wg == 0 && part == 0,
+            epi_up<C, C::EPI_COLS, CAL>(a, par, C::QB, C::QS + part * C::COUT, dcol, wg * C::EPI_COLS, e, p, valid, wg == 0 && part == 0,
                                    part * (C::COUT / C::CUP));
             tc_fence_before();
             mbar_arrive(&tempty[b]);
             continue;
         }
         if constexpr (C::EPI == EPI_UP) {   // one warpgroup: conv, then the ConvT
-            if (!epi_conv<C, C::COUT, CAL>(a, smem, sbias, scs, dcol, 0, ab, e, p, m, valid, sx,
+            if (!epi_conv<C, C::COUT, CAL>(a, smem, par, C::QB, C::QS, dcol, 0, ab, e, p, m, valid, sx,
                                       a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
                                       (uint32_t)(i >> 1) * C::xchunks(C::COUT), abort))
                 return false;
@@ -831,11 +835,11 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
             mbar_arrive(&a2full[ab]);
             if (!mbar_wait(&t2full[b], ph_b, abort)) return false;
             tc_fence_after();
-            epi_up<C, C::N2, CAL>(a, sbias2, scs2, dcol, 0, e, p, valid, true);
+            epi_up<C, C::N2, CAL>(a, par, C::QB2, C::QS2, dcol, 0, e, p, valid, true);
         } else {                            // this warpgroup's conv columns
             static_assert(!C::PAIRED || C::EPI == EPI_STORE, "paired stores");
             // paired taps (the wide network's split dec3): E[m] + O[m + 1]
-            if (!epi_conv<C, C::EPI_COLS, CAL>(a, smem, sbias, scs, dcol, wg * C::EPI_COLS, ab, e, p, m, valid, sx, 0,
+            if (!epi_conv<C, C::EPI_COLS, CAL>(a, smem, par, C::QB + part * C::COUT, C::QS + part * C::COUT, dcol, wg * C::EPI_COLS, ab, e, p, m, valid, sx, 0,
                                           inseq, &xready[ab], (uint32_t)(i >> 1) * C::xchunks(C::EPI_COLS), abort))
                 return false;
             if (wg == 0 && (p == 0 || p == C::L - 1)) {
@@ -864,7 +868,8 @@ __device__ bool epilogue(const TcArgs &a, unsigned char *smem, uint64_t *bar, ui
 }
 
 template <class C, bool CAL>
-__global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(TcArgs a) {
+__global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG)
+k_conv_tc(TcArgs a, const __grid_constant__ ParBlock<C::NPAR> par) {
     using B = Bars<C>;
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + C::OFF_BAR);
@@ -873,17 +878,6 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
     volatile int *ring = reinterpret_cast<volatile int *>(reinterpret_cast<unsigned char *>(bar) + B::RING_OFF);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    // biases, column scales and the final conv in shared memory
-    float *par = reinterpret_cast<float *>(smem + C::OFF_PAR);
-    const int part = (int)blockIdx.x % C::NSPLIT;   // this CTA's part of a split layer
-    for (int k = threadIdx.x; k < C::NPAR; k += C::THREADS) {
-        float v;
-        if (k < C::COUT) v = C::EPI == EPI_CONVT ? a.bias[k % C::CUP] : a.bias[part * C::COUT + k];
-        else if (k < C::COUT + C::N2) v = a.bias2[(k - C::COUT) % (C::CUP > 0 ? C::CUP : 1)];
-        else if (k < 2 * C::COUT + C::N2) v = a.cs ? a.cs[part * C::COUT + k - C::COUT - C::N2] : 1.0f;
-        else v = a.cs2 ? a.cs2[k - 2 * C::COUT - C::N2] : 1.0f;
-        par[k] = v;
-    }
     if (threadIdx.x == 0) {
         mbar_init(&bar[B::W], 1);
         for (int s = 0; s < C::STAGES; ++s) {
@@ -932,7 +926,7 @@ __global__ void __launch_bounds__(C::THREADS) __maxnreg__(C::MAXREG) k_conv_tc(T
         // 97 us per 1000 events, FP8 dec2_up1 57 -> 60): they keep the plain one-thread branch.
         if (C::NSPLIT > 1 ? elect_one() : lane == 0) ok = mma_issuer<C>(r, smem, bar, tmem, ring, abort);
     } else {
-        ok = epilogue<C, CAL>(r, smem, bar, tmem, ring, abort, warp, lane);
+        ok = epilogue<C, CAL>(r, par, smem, bar, tmem, ring, abort, warp, lane);
     }
     if (!ok) {
         *abort = 1;
@@ -987,7 +981,12 @@ cudaError_t launch_conv(const TcArgs &a, cudaStream_t s, const ProfHook *prof, c
     grid = grid / C::NSPLIT * C::NSPLIT;             // every part gets the same CTAs
     if (grid < C::NSPLIT) grid = C::NSPLIT;
     ProfScope ps(prof, name, s);
-    return launch_pdl(k_conv_tc<C, CAL>, dim3(grid), dim3(C::THREADS), (size_t)smem, s, a);
+    ParBlock<C::NPAR> par;
+    par.set(C::QB, a.bias, C::NBIAS);
+    if (C::N2) par.set(C::QB2, a.bias2, C::CUP);
+    par.set(C::QS, a.cs, C::NSC);
+    par.set(C::QS2, a.cs2, C::NSC2);
+    return launch_pdl(k_conv_tc<C, CAL>, dim3(grid), dim3(C::THREADS), (size_t)smem, s, a, par);
 }
 
 // ---------------------------------------------------------------- weight packing (host)
@@ -1188,6 +1187,7 @@ bool tc_pack_weights(int precision, const std::vector<LayerF32> &layers, const f
         off_w[li] = pk.put_raw(img.data(), img.size());
         const size_t nbias = up ? Lw.shape[1] : Lw.shape[0];
         off_b[li] = pk.put_raw(Lw.b, nbias * sizeof(float));
+        std::copy(Lw.b, Lw.b + nbias, net->hb[li]);
         // fp8 dequantisation scale per accumulator column: input activation scale x weight scale
         std::vector<float> cs(cout, 1.0f);
         if (precision == PVF_FP8_E4M3) {
@@ -1197,6 +1197,7 @@ bool tc_pack_weights(int precision, const std::vector<LayerF32> &layers, const f
             for (int c = 0; c < cout; ++c) cs[c] = act_scale[in_idx[li]] * scale[c];
         }
         off_s[li] = pk.put_raw(cs.data(), cs.size() * sizeof(float));
+        std::copy(cs.begin(), cs.end(), net->hs[li]);
     }
     // FC images (f16 in the FP16 form, bf16 in the others): element (out o, in i) of layer l at
     // ((i / 8) * R + row) * 16 + (i % 8) * 2 of the layer's image, R rows per plane;
@@ -1239,7 +1240,7 @@ static cudaError_t run_tc(const TcNet &n, const UnetBuffers &b, int ne, const in
                           cudaStream_t s, const ProfHook *prof) {
     const float *sc = n.act_scale;
     auto inv = [&](int i) { return is16(PREC) ? 1.0f : 1.0f / sc[i]; };
-    auto cs = [&](int li) { return is16(PREC) ? nullptr : n.wscale[li]; };
+    auto cs = [&](int li) { return is16(PREC) ? nullptr : li == 5 ? n.wscale[li] : n.hs[li]; };
     auto W = [&](int li) { return static_cast<const unsigned char *>(n.w[li]); };
     auto U = [](void *p) { return static_cast<unsigned char *>(p); };
     cudaError_t err;
@@ -1255,17 +1256,17 @@ static cudaError_t run_tc(const TcNet &n, const UnetBuffers &b, int ne, const in
     // enc2: p1 (s0) -> e2, p2 (s1)
     EncArgs g;
     a.inA = U(b.s0); a.inB = nullptr; a.out = U(b.e2); a.outp = U(b.s1);
-    a.w = W(0); a.bias = n.b[0]; a.cs = cs(0); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
+    a.w = W(0); a.bias = n.hb[0]; a.cs = cs(0); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
     if constexpr (N::FUSED_ENC) g.c2 = a;
     else if ((err = launch_conv<typename N::Enc2>(a, s, prof, "enc2", n.ctas_per_sm[0])) != cudaSuccess) return err;
     // enc3: p2 (s1) -> e3, p3 (s0)
     a.inA = U(b.s1); a.out = U(b.e3); a.outp = U(b.s0); a.sched = sched(1);
-    a.w = W(1); a.bias = n.b[1]; a.cs = cs(1); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
+    a.w = W(1); a.bias = n.hb[1]; a.cs = cs(1); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
     if constexpr (N::FUSED_ENC) g.c3 = a;
     else if ((err = launch_conv<typename N::Enc3>(a, s, prof, "enc3", n.ctas_per_sm[1])) != cudaSuccess) return err;
     // enc4 + up3: p3 (s0) -> u3 (up)
     a.inA = U(b.s0); a.out = U(b.up); a.outp = nullptr; a.sched = sched(2);
-    a.w = W(2); a.bias = n.b[2]; a.cs = cs(2); a.w2 = W(6); a.bias2 = n.b[6]; a.cs2 = cs(6);
+    a.w = W(2); a.bias = n.hb[2]; a.cs = cs(2); a.w2 = W(6); a.bias2 = n.hb[6]; a.cs2 = cs(6);
     a.mid_inv = inv(kScaleE4); a.out_inv = inv(kScaleL3); a.amax_mid = kScaleE4; a.amax_out = kScaleL3;
     if constexpr (N::FUSED_ENC) {      // the three layers in one kernel; p2 and p3 stay in shared memory
         g.c4 = a;
@@ -1275,12 +1276,12 @@ static cudaError_t run_tc(const TcNet &n, const UnetBuffers &b, int ne, const in
     }
     // dec3 + up2: [u3 (up), e3] -> u2 (deep)
     a.inA = U(b.up); a.inB = U(b.e3); a.out = U(b.deep); a.sched = sched(3);
-    a.w = W(3); a.bias = n.b[3]; a.cs = cs(3); a.w2 = W(7); a.bias2 = n.b[7]; a.cs2 = cs(7);
+    a.w = W(3); a.bias = n.hb[3]; a.cs = cs(3); a.w2 = W(7); a.bias2 = n.hb[7]; a.cs2 = cs(7);
     a.mid_inv = inv(kScaleD3); a.out_inv = inv(kScaleL2); a.amax_mid = kScaleD3; a.amax_out = kScaleL2;
     if ((err = launch_conv<typename N::Dec3Up2>(a, s, prof, "dec3_up2", n.ctas_per_sm[3])) != cudaSuccess) return err;
     // dec2 + up1: [u2 (deep), e2] -> u1 (up)
     a.inA = U(b.deep); a.inB = U(b.e2); a.out = U(b.up); a.sched = sched(4);
-    a.w = W(4); a.bias = n.b[4]; a.cs = cs(4); a.w2 = W(8); a.bias2 = n.b[8]; a.cs2 = cs(8);
+    a.w = W(4); a.bias = n.hb[4]; a.cs = cs(4); a.w2 = W(8); a.bias2 = n.hb[8]; a.cs2 = cs(8);
     a.mid_inv = inv(kScaleD2); a.out_inv = inv(kScaleL1); a.amax_mid = kScaleD2; a.amax_out = kScaleL1;
     if ((err = launch_conv<typename N::Dec2Up1>(a, s, prof, "dec2_up1", n.ctas_per_sm[4])) != cudaSuccess) return err;
     // dec1 + final conv: [u1 (up), e1] -> logits (float32)
@@ -1298,7 +1299,7 @@ static cudaError_t run_tc32(const TcNet &n, const UnetBuffers &b, int ne, const 
     using N = Net32<PREC>;
     const float *sc = n.act_scale;
     auto inv = [&](int i) { return is16(PREC) ? 1.0f : 1.0f / sc[i]; };
-    auto cs = [&](int li) { return is16(PREC) ? nullptr : n.wscale[li]; };
+    auto cs = [&](int li) { return is16(PREC) ? nullptr : li == 5 ? n.wscale[li] : n.hs[li]; };
     auto W = [&](int li) { return static_cast<const unsigned char *>(n.w[li]); };
     auto U = [](void *p) { return static_cast<unsigned char *>(p); };
     cudaError_t err;
@@ -1312,31 +1313,31 @@ static cudaError_t run_tc32(const TcNet &n, const UnetBuffers &b, int ne, const 
     // enc2: p1 (s0) -> e2, p2 (s1)
     a.sched = sched(0);
     a.inA = U(b.s0); a.inB = nullptr; a.out = U(b.e2); a.outp = U(b.s1);
-    a.w = W(0); a.bias = n.b[0]; a.cs = cs(0); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
+    a.w = W(0); a.bias = n.hb[0]; a.cs = cs(0); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
     if ((err = launch_conv<typename N::Enc2>(a, s, prof, "enc2", n.ctas_per_sm[0])) != cudaSuccess) return err;
     // enc3: p2 (s1) -> e3, p3 (s0)
     a.inA = U(b.s1); a.out = U(b.e3); a.outp = U(b.s0); a.sched = sched(1);
-    a.w = W(1); a.bias = n.b[1]; a.cs = cs(1); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
+    a.w = W(1); a.bias = n.hb[1]; a.cs = cs(1); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
     if ((err = launch_conv<typename N::Enc3>(a, s, prof, "enc3", n.ctas_per_sm[1])) != cudaSuccess) return err;
     // enc4 (split): p3 (s0) -> e4 (deep)
     a.inA = U(b.s0); a.out = U(b.deep); a.outp = nullptr; a.sched = sched(2);
-    a.w = W(2); a.bias = n.b[2]; a.cs = cs(2); a.out_inv = inv(kScaleE4); a.amax_out = kScaleE4;
+    a.w = W(2); a.bias = n.hb[2]; a.cs = cs(2); a.out_inv = inv(kScaleE4); a.amax_out = kScaleE4;
     if ((err = launch_conv<typename N::Enc4>(a, s, prof, "enc4", n.ctas_per_sm[2])) != cudaSuccess) return err;
     // up3 (ConvT GEMM, split by r): e4 (deep) -> u3 (up)
     a.inA = U(b.deep); a.out = U(b.up);
-    a.w = W(6); a.bias = n.b[6]; a.cs = cs(6); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
+    a.w = W(6); a.bias = n.hb[6]; a.cs = cs(6); a.out_inv = inv(kScaleL3); a.amax_out = kScaleL3;
     if ((err = launch_conv<typename N::Up3>(a, s, prof, "up3", n.ctas_per_sm[2])) != cudaSuccess) return err;
     // dec3 (split): [u3 (up), e3] -> d3 (deep)
     a.inA = U(b.up); a.inB = U(b.e3); a.out = U(b.deep); a.sched = sched(3);
-    a.w = W(3); a.bias = n.b[3]; a.cs = cs(3); a.out_inv = inv(kScaleD3); a.amax_out = kScaleD3;
+    a.w = W(3); a.bias = n.hb[3]; a.cs = cs(3); a.out_inv = inv(kScaleD3); a.amax_out = kScaleD3;
     if ((err = launch_conv<typename N::Dec3>(a, s, prof, "dec3", n.ctas_per_sm[3])) != cudaSuccess) return err;
     // up2 (ConvT GEMM): d3 (deep) -> u2 (up)
     a.inA = U(b.deep); a.inB = nullptr; a.out = U(b.up);
-    a.w = W(7); a.bias = n.b[7]; a.cs = cs(7); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
+    a.w = W(7); a.bias = n.hb[7]; a.cs = cs(7); a.out_inv = inv(kScaleL2); a.amax_out = kScaleL2;
     if ((err = launch_conv<typename N::Up2>(a, s, prof, "up2", n.ctas_per_sm[3])) != cudaSuccess) return err;
     // dec2 + up1: [u2 (up), e2] -> u1 (deep)
     a.inA = U(b.up); a.inB = U(b.e2); a.out = U(b.deep); a.sched = sched(4);
-    a.w = W(4); a.bias = n.b[4]; a.cs = cs(4); a.w2 = W(8); a.bias2 = n.b[8]; a.cs2 = cs(8);
+    a.w = W(4); a.bias = n.hb[4]; a.cs = cs(4); a.w2 = W(8); a.bias2 = n.hb[8]; a.cs2 = cs(8);
     a.mid_inv = inv(kScaleD2); a.out_inv = inv(kScaleL1); a.amax_mid = kScaleD2; a.amax_out = kScaleL1;
     if ((err = launch_conv<typename N::Dec2Up1>(a, s, prof, "dec2_up1", n.ctas_per_sm[4])) != cudaSuccess)
         return err;
@@ -1359,18 +1360,18 @@ static cudaError_t stall_tc(const TcNet &n, const UnetBuffers &b, int ne, uint32
     a.out = static_cast<unsigned char *>(b.e2);
     a.outp = static_cast<unsigned char *>(b.s1);
     a.w = static_cast<const unsigned char *>(n.w[0]);
-    a.bias = n.b[0];
-    a.cs = is16(PREC) ? nullptr : n.wscale[0];
+    a.bias = n.hb[0];
+    a.cs = is16(PREC) ? nullptr : n.hs[0];
     a.out_inv = is16(PREC) ? 1.0f : 1.0f / n.act_scale[kScaleL2];
     a.stall_test_us = stall_us;
     EncArgs g;
     g.c2 = g.c3 = g.c4 = a;
     g.c3.w = static_cast<const unsigned char *>(n.w[1]);
-    g.c3.bias = n.b[1];
+    g.c3.bias = n.hb[1];
     g.c4.w = static_cast<const unsigned char *>(n.w[2]);
-    g.c4.bias = n.b[2];
+    g.c4.bias = n.hb[2];
     g.c4.w2 = static_cast<const unsigned char *>(n.w[6]);
-    g.c4.bias2 = n.b[6];
+    g.c4.bias2 = n.hb[6];
     return launch_enc<N>(g, s, nullptr);
 }
 

@@ -33,6 +33,8 @@ struct TcNet {
     const void *w[9];        // enc2, enc3, enc4, dec3, dec2, dec1, up3, up2, up1 (packed)
     const float *b[9];       // biases, float32
     const float *wscale[9];  // per-accumulator-column dequantisation scales (fp8)
+    // the same two on the host: the conv kernels take them as launch parameters
+    float hb[9][8 * kC0Max], hs[9][8 * kC0Max];
     float act_scale[PVF_N_ACT_SCALES];
     const float *final_w;    // final conv (float32, W[t][ci] then b)
     const unsigned char *fc_img;   // bf16 FC operand images (kFcImgBytes)
