@@ -306,13 +306,17 @@ __device__ __forceinline__ void enc_epi(const EncPool &L, const P &par, const Tc
             }
             if (valid) w = make_uint4(x[0], x[1], x[2], x[3]);
         } else {
-            if (st) put16<PREC>(dst, 0, v, L.out_inv);
+            uint32_t r[4];
+            pack_e4m3<16>(v, L.out_inv, r);
+            if (st) *reinterpret_cast<uint4 *>(dst) = make_uint4(r[0], r[1], r[2], r[3]);
             dst += L.plane;
-            float x[8];
+            uint32_t x[2];
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                x[q] = fmaxf(odd ? v[8 + q] : v[q], __shfl_xor_sync(0xffffffffu, odd ? v[q] : v[8 + q], 1));
-            if (valid) pack_e4m3<8>(x, L.out_inv, reinterpret_cast<uint32_t *>(&w));
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? r[q] : r[2 + q], 1);
+                x[q] = max4_e4m3(odd ? r[2 + q] : r[q], got);
+            }
+            if (valid) w = make_uint4(x[0], x[1], 0, 0);
         }
         constexpr uint32_t STEP = (is16(PREC) ? 2 : 1) * PLANE;        // planes of 16 channels
         auto put = [&](uint32_t to, uint4 q) {

@@ -665,14 +665,20 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
                                 make_uint4(w[0], w[1], w[2], w[3]);
                     }
                 } else {
-                    if (valid) put16<C::PREC>(dst, (size_t)C::ROWS_E * 16, v, a.out_inv);
-                    if constexpr (C::EPI == EPI_POOL) {
-                        float w[16];
+                    uint32_t r[4];
+                    pack_e4m3<16>(v, a.out_inv, r);
+                    if (valid) *reinterpret_cast<uint4 *>(dst) = make_uint4(r[0], r[1], r[2], r[3]);
+                    if constexpr (C::EPI == EPI_POOL) {      // likewise, half a plane's row each
+                        const bool odd = (m & 1) != 0;
+                        uint32_t w[2];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) w[j] = fmaxf(v[j], __shfl_xor_sync(0xffffffffu, v[j], 1));
-                        if (valid && inseq && (m & 1) == 0)
-                            put16<C::PREC>(a.outp + planar_off(e, c0 / C::PW, C::POUT, ROWS_P, prow),
-                                           (size_t)ROWS_P * 16, w, a.out_inv);
+                        for (int j = 0; j < 2; ++j) {
+                            const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? r[j] : r[2 + j], 1);
+                            w[j] = max4_e4m3(odd ? r[2 + j] : r[j], got);
+                        }
+                        if (valid && inseq)
+                            *reinterpret_cast<uint2 *>(a.outp + planar_off(e, c0 / C::PW, C::POUT, ROWS_P, prow) +
+                                                       (odd ? 8 : 0)) = make_uint2(w[0], w[1]);
                     }
                 }
             }

@@ -223,13 +223,27 @@ __device__ __forceinline__ void pack_e4m3(const float *v, float inv_scale, uint3
     static_assert(N % 4 == 0, "whole words");
 #pragma unroll
     for (int i = 0; i < N; i += 4) {
+        const float2 sc = make_float2(inv_scale, inv_scale);
         const __nv_fp8x2_storage_t lo =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[i] * inv_scale, v[i + 1] * inv_scale), __NV_SATFINITE, __NV_E4M3);
+            __nv_cvt_float2_to_fp8x2(__fmul2_rn(make_float2(v[i], v[i + 1]), sc), __NV_SATFINITE, __NV_E4M3);
         const __nv_fp8x2_storage_t hi =
-            __nv_cvt_float2_to_fp8x2(make_float2(v[i + 2] * inv_scale, v[i + 3] * inv_scale), __NV_SATFINITE,
-                                     __NV_E4M3);
+            __nv_cvt_float2_to_fp8x2(__fmul2_rn(make_float2(v[i + 2], v[i + 3]), sc), __NV_SATFINITE, __NV_E4M3);
         out[i / 4] = (uint32_t)lo | ((uint32_t)hi << 16);
     }
+}
+
+// The larger of four pairs of e4m3 codes (the other code where one is a NaN). Rounding is
+// monotonic, so this is the code of the larger value; f16 holds every e4m3 value, so the way
+// through it is exact.
+__device__ __forceinline__ uint32_t max4_e4m3(uint32_t a, uint32_t b) {
+    uint32_t out = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const __half2 x = __half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(a >> (16 * h)), __NV_E4M3));
+        const __half2 y = __half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(b >> (16 * h)), __NV_E4M3));
+        out |= (uint32_t)__nv_cvt_halfraw2_to_fp8x2(__half2_raw(__hmax2(x, y)), __NV_SATFINITE, __NV_E4M3) << (16 * h);
+    }
+    return out;
 }
 
 // ---------------------------------------------------------------- kernel arguments
