@@ -150,16 +150,25 @@ __device__ __forceinline__ void validate_sort(const FrontArgs &a, int ge, int ti
         sslice[t] = s < 0 ? 255 : (uint8_t)(s | (tag << 6));
     }
     __syncthreads();
-    if (tid == 0) {
-        int acc = 0;
-        for (int s = 0; s < kSlices; ++s) { sseg[s] = acc; acc += scnt[s]; }
-        sseg[kSlices] = acc;
-    }
-    __syncthreads();
-    // stable ranks by slice: warp 0 walks the tracks in input order, once for their own
-    // slices and once more for the second slices of boundary tracks
+    // warp 0: the slices' bounds (a scan with two slices per lane; one thread adding them up took
+    // 1400 cycles), then stable ranks by slice, walking the tracks in input order, once for their
+    // own slices and once more for the second slices of boundary tracks
     if (tid < 32) {
         const unsigned lane = tid;
+        static_assert(kSlices % 2 == 0 && kSlices <= 64, "two slices per lane");
+        const int a0 = scnt[2 * lane < kSlices ? 2 * lane : kSlices], a1 = scnt[2 * lane < kSlices ? 2 * lane + 1 : kSlices];
+        int incl = a0 + a1;          // scnt[kSlices] is 0
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((int)lane >= o) incl += y;
+        }
+        if (2 * lane < kSlices) {
+            sseg[2 * lane] = incl - a0 - a1;
+            sseg[2 * lane + 1] = incl - a1;
+        }
+        if (lane == 31) sseg[kSlices] = incl;
+        __syncwarp();
 #pragma unroll 1
         for (int pass = 0; pass < (EDGE ? 2 : 1); ++pass) {
             for (int base = 0; base < n; base += 32) {
@@ -227,18 +236,18 @@ __device__ __forceinline__ void store_half8(void *base, int64_t e, int64_t rows_
 // Thread tid owns channels [8 h, 8 h + 8), h = tid & 1, of every position pair it takes,
 // so its 40 weights and 8 biases stay in registers and the loop reads only the histogram
 // from shared memory; the two threads of a pair write the two halves of each row.
-// IV: the per-interval layout of the tensor-core forms: e1 and p1 hold the event's kSlices
+// This is the per-interval layout of the tensor-core forms: e1 and p1 hold the event's kSlices
 // sequences end to end, each the conv of the interval's kIvLen-bin window (its bins with
 // kIvPad zero bins on each side), two zero rows before each sequence and two after the
 // last (neighbouring sequences share the two between them).
-template <class T, int NT, bool AMAX, bool IV = false>
+template <class T, int NT, bool AMAX>
 __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, const float *shist,
                                             const float *senc) {
     static_assert(NT % 2 == 0, "thread pairs");
     constexpr int S1 = kIvLen + kPad, S2 = kIvLen / 2 + kPad;   // rows per sequence
-    constexpr int RQ = quad_rows(IV ? kSlices * S1 - kPad : kBins);     // e1: the quad layout
-    const int64_t rows2 = IV ? (int64_t)kSlices * S2 + kPad : padded_rows(kBins / 2);
-    constexpr int NQ = IV ? kSlices * (kIvLen / 2) : kBins / 2;         // position pairs
+    constexpr int RQ = quad_rows(kSlices * S1 - kPad);     // e1: the quad layout
+    constexpr int64_t rows2 = (int64_t)kSlices * S2 + kPad;
+    constexpr int NQ = kSlices * (kIvLen / 2);         // position pairs
     const float inv = a.e1_inv_scale;
     const int h = tid & 1;
     float w[5][8], bias[8];
@@ -251,20 +260,15 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
     float vmax = 0.0f;
 #pragma unroll 2   // two position pairs in flight per thread: front 81.6 -> 79.5 us (FP16)
     for (int qi = tid >> 1; qi < NQ; qi += NT / 2) {
-        // the pair's sequence (IV) and first position; e1 positions p1, p1 + 1, p1 row r2
-        const int sq = IV ? qi / (kIvLen / 2) : 0, q = IV ? qi % (kIvLen / 2) : qi;
-        const int p1 = sq * S1 * IV + 2 * q;
-        const int64_t r2 = (int64_t)sq * S2 * IV + q + kPad;
+        // the pair's sequence and first position; e1 positions p1, p1 + 1, p1 row r2
+        const int sq = qi / (kIvLen / 2), q = qi % (kIvLen / 2);
+        const int p1 = sq * S1 + 2 * q;
+        const int64_t r2 = (int64_t)sq * S2 + q + kPad;
         float hv[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            if constexpr (IV) {
-                const int b = 2 * q + k - 2 - kIvPad;    // bin of the interval at window position
-                hv[k] = (b >= 0 && b < kSliceBins) ? shist[sq * kSliceBins + b] : 0.0f;
-            } else {
-                const int p = 2 * q + k - 2;
-                hv[k] = (p >= 0 && p < kBins) ? shist[p] : 0.0f;
-            }
+            const int b = 2 * q + k - 2 - kIvPad;    // bin of the interval at window position
+            hv[k] = (b >= 0 && b < kSliceBins) ? shist[sq * kSliceBins + b] : 0.0f;
         }
         float v0[8], v1[8];
         // channel pairs (j, j + 1) as one packed two-lane FMA (each lane an fmaf, in the
@@ -314,16 +318,92 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
         for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
         if ((tid & 31) == 0) atomicMax(reinterpret_cast<int *>(a.amax), __float_as_int(vmax));
     }
-    if constexpr (IV) {     // the two rows before each sequence and the two after the last
-        for (int idx = tid; idx < (kSlices + 1) * 2; idx += NT) {
-            const int sq = idx >> 1, k = idx & 1;
-            zero_quad<T, kC0>(a.e1, e, RQ, sq * S1 + k - kPad);
-            zero_row16<T>(a.p1, e, rows2, (int64_t)sq * S2 + k);
+    for (int idx = tid; idx < (kSlices + 1) * 2; idx += NT) {   // the two rows before each sequence and after the last
+        const int sq = idx >> 1, k = idx & 1;
+        zero_quad<T, kC0>(a.e1, e, RQ, sq * S1 + k - kPad);
+        zero_row16<T>(a.p1, e, rows2, (int64_t)sq * S2 + k);
+    }
+}
+
+// The same for whole events of the tensor-core forms, four positions per step: they share their
+// eight histogram bins (shist is zero for two bins on either side), their addresses (one row of
+// the four residue planes of e1, two rows of p1) and, in registers, the weights of the thread's 8
+// channels. Same arithmetic per position as enc1_pool_t.
+template <class T, int NT, bool AMAX>
+__device__ __forceinline__ void enc1_pool_quads(const FrontArgs &a, int e, int tid, const float *shist,
+                                                const float *senc) {
+    static_assert(sizeof(T) <= 2 && kBins % 4 == 0, "plane-major forms");
+    constexpr int RQ = quad_rows(kBins);
+    constexpr int P = kC0 * (int)sizeof(T) / 16;                          // planes: 2, or 1 of e4m3
+    const int64_t rows2 = padded_rows(kBins / 2);
+    const float inv = a.e1_inv_scale;
+    const int h = tid & 1;
+    float2 w[5][4], bias[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int t = 0; t < 5; ++t) w[t][j] = make_float2(senc[t * kC0 + 8 * h + 2 * j], senc[t * kC0 + 8 * h + 2 * j + 1]);
+        bias[j] = make_float2(senc[5 * kC0 + 8 * h + 2 * j], senc[5 * kC0 + 8 * h + 2 * j + 1]);
+    }
+    float vmax = 0.0f;
+    constexpr int half = sizeof(T) == 2 ? 0 : 8;                          // e4m3: half a plane's row per thread
+    unsigned char *e1 = reinterpret_cast<unsigned char *>(a.e1) + quad_off(e, P == 2 ? h : 0, P, RQ, 0) + half * h;
+    unsigned char *p1 = reinterpret_cast<unsigned char *>(a.p1) + planar_off(e, P == 2 ? h : 0, P, rows2, kPad) + half * h;
+#pragma unroll 1
+    for (int q = tid >> 1; q < kBins / 4; q += NT / 2) {
+        float hv[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 x = *reinterpret_cast<const float2 *>(shist + 4 * q - 2 + 2 * k);
+            hv[2 * k] = x.x;
+            hv[2 * k + 1] = x.y;
         }
-    } else if (tid < 4) {
+        float v[4][8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float2 acc = bias[j];
+#pragma unroll
+                for (int t = 0; t < 5; ++t) acc = __ffma2_rn(w[t][j], make_float2(hv[i + t], hv[i + t]), acc);
+                acc = leaky2(acc);
+                v[i][2 * j] = acc.x;
+                v[i][2 * j + 1] = acc.y;
+                if constexpr (AMAX) vmax = fmaxf(vmax, fmaxf(fabsf(acc.x), fabsf(acc.y)));
+            }
+        if constexpr (sizeof(T) == 2) {
+            uint4 r[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                r[i] = pack8<T>(v[i]);
+                *reinterpret_cast<uint4 *>(e1 + (size_t)(i * RQ + q) * 16) = r[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)     // the maximum of the rounded values is the rounded maximum
+                *reinterpret_cast<uint4 *>(p1 + (size_t)(2 * q + i) * 16) =
+                    make_uint4(max2<T>(r[2 * i].x, r[2 * i + 1].x), max2<T>(r[2 * i].y, r[2 * i + 1].y),
+                               max2<T>(r[2 * i].z, r[2 * i + 1].z), max2<T>(r[2 * i].w, r[2 * i + 1].w));
+        } else {
+            uint2 r[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                pack_e4m3<8>(v[i], inv, reinterpret_cast<uint32_t *>(&r[i]));
+                *reinterpret_cast<uint2 *>(e1 + (size_t)(i * RQ + q) * 16) = r[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                *reinterpret_cast<uint2 *>(p1 + (size_t)(2 * q + i) * 16) =
+                    make_uint2(max4_e4m3(r[2 * i].x, r[2 * i + 1].x), max4_e4m3(r[2 * i].y, r[2 * i + 1].y));
+        }
+    }
+    if constexpr (AMAX) {   // calibration: integer max on the float bits (order-independent)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+        if ((tid & 31) == 0) atomicMax(reinterpret_cast<int *>(a.amax), __float_as_int(vmax));
+    }
+    if (tid < 4) {
         zero_quad<T, kC0>(a.e1, e, RQ, tid < 2 ? tid - kPad : kBins + tid - kPad);   // -2, -1 and L, L + 1
-        const int rp = tid < 2 ? tid : kBins / 2 + tid;
-        zero_row16<T>(a.p1, e, rows2, rp);
+        zero_row16<T>(a.p1, e, rows2, tid < 2 ? tid : kBins / 2 + tid);
     }
 }
 
@@ -477,8 +557,13 @@ __device__ __forceinline__ void enc1_pool(const FrontArgs &a, int e, int tid, co
                                           const float *senc) {
     if constexpr (REGW) {
         static_assert(C0 == kC0, "register weights for width 16");
-        if (a.amax) enc1_pool_t<T, NT, true, IV>(a, e, tid, shist, senc);
-        else enc1_pool_t<T, NT, false, IV>(a, e, tid, shist, senc);
+        if constexpr (IV) {
+            if (a.amax) enc1_pool_t<T, NT, true>(a, e, tid, shist, senc);
+            else enc1_pool_t<T, NT, false>(a, e, tid, shist, senc);
+        } else {
+            if (a.amax) enc1_pool_quads<T, NT, true>(a, e, tid, shist, senc);
+            else enc1_pool_quads<T, NT, false>(a, e, tid, shist, senc);
+        }
     } else {
         if (a.amax) enc1_pool_shared_t<T, NT, true, C0>(a, e, tid, shist, senc);
         else enc1_pool_shared_t<T, NT, false, C0>(a, e, tid, shist, senc);

@@ -43,8 +43,9 @@ template <int NT> struct TcSmem {
     static constexpr size_t enc1 = bias + sizeof(float) * kFcBTotal;   // kEnc1Floats
     static constexpr size_t x = (enc1 + sizeof(float) * kEnc1FloatsMax + 127) / 128 * 128;  // 2 planes x NT rows
     static constexpr size_t h = x + 2 * kPlane;                        // 4 planes x NT rows
-    static constexpr size_t hist = h + 4 * kPlane;
-    static constexpr size_t cnt = hist + sizeof(float) * kBins;
+    // the histogram, with four zero floats on either side (enc1 reads two bins past its ends)
+    static constexpr size_t hist = h + 4 * kPlane + 16;
+    static constexpr size_t cnt = hist + sizeof(float) * kBins + 16;
     static constexpr size_t seg = cnt + sizeof(int) * 48;
     static constexpr size_t run = seg + sizeof(int) * 48;
     static constexpr size_t bar = (run + sizeof(int) * 48 + 15) / 16 * 16;   // mbarrier, TMEM slot, flag, next event
@@ -72,7 +73,9 @@ template <> struct FcOp<PVF_FP16> {
 // 1 + u to 1.
 __device__ __forceinline__ float softplus_tc(float x) {
     const float u = __expf(-fabsf(x));
-    const float l = fmaf(__log2f(1.0f + u), 0.69314718f, fmaxf(x, 0.0f));
+    float lg;      // 1 + u is in [1, 2]: the flush-to-zero form gives the same without scaling for denormals
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(1.0f + u));
+    const float l = fmaf(lg, 0.69314718f, fmaxf(x, 0.0f));
     return x < -15.0f ? u : l;
 }
 
@@ -120,6 +123,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
         *never = 0;
         fence_mbar_init();
     }
+    if (tid < 8) shist[tid < 4 ? tid - 4 : kBins + tid - 4] = 0.0f;
     if (warp == 0) {
         tmem_alloc(tmem_slot, kTmemCols);
         tmem_relinquish();
@@ -128,8 +132,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    // launched in stream order (its inputs come from the caller); lets the next kernel
-    // start its prologue while this one runs
+    // The prologue above read the handle's weights only. The caller's inputs, and the buffers that
+    // earlier calls' kernels may still read, are touched after the previous kernel of the stream has
+    // finished (back to back, its tail hides this launch and prologue); then the next kernel may
+    // start its own prologue.
+    grid_dep_wait();
     grid_dep_launch();
     const uint32_t img = smem_u32(smem + TcSmem::img);
     const uint32_t sx = smem_u32(smem + TcSmem::x), sh = smem_u32(smem + TcSmem::h);
@@ -163,10 +170,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
             if (failed) nvalid = 0;        // a timed-out MMA ends the tensor-core work
             for (int c0 = 0; c0 < nvalid && !failed; c0 += kPass) {
                 const int ntile = NT == 128 ? 1 : (nvalid - c0 > kRows ? 2 : 1);
-                const bool active = g < ntile;         // warpgroup has a tile in this pass
                 const int r = c0 + g * kRows + m;
                 const bool live = r < nvalid;
-                if (active) {   // X row: the track's features in 16 bits, zero rows past the event
+                const int nrow = min(nvalid - c0, kPass);
+                if (g * kRows + (m & ~31) < nrow) {   // X row: the track's features in 16 bits, zero rows past the event
                     float x[16];
 #pragma unroll
                     for (int k = 0; k < 16; ++k) x[k] = 0.0f;
@@ -180,7 +187,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
                 fence_proxy_async_smem();
                 tc_fence_before();
                 __syncthreads();
-                const int nrow = min(nvalid - c0, kPass);
                 const int n6 = (nrow + 15) / 16 * 16;          // output MMA: N = tracks, rounded
                 for (int l = 0; l < 6 && !failed; ++l) {
                     tc_fence_after();
@@ -214,7 +220,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
                     if (__syncthreads_or(!ok)) { failed = true; break; }
                     tc_fence_after();
                     if (l < 5) {
-                        if (active) {
+                        // a warp whose 32 rows lie past the pass's tracks leaves its rows as they are:
+                        // no other row depends on them, and the output layer reads none of them
+                        if (g * kRows + (m & ~31) < nrow) {
                             float v[32];
                             tmem_ld16(dcol, *reinterpret_cast<float(*)[16]>(v));
                             tmem_ld16(dcol + 16, *reinterpret_cast<float(*)[16]>(v + 16));
@@ -255,9 +263,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
                                 for (int t = 0; t < 32; ++t) acc = __fadd_rn(acc, v[t]);
                                 continue;
                             }
-                            // several segments in this chunk: one branch-free masked pass per
-                            // segment, in row order (adding zeros leaves the sum bit-identical,
-                            // and the loop body stays small enough for the instruction cache)
+                            // several segments in this chunk: per segment, in row order, the groups of
+                            // 8 rows that it touches, masked where it holds part of one (leaving out
+                            // or adding zeros leaves the sum bit-identical, and the loop body stays
+                            // small enough for the instruction cache)
                             const int cnt = min(32, ce - col);
                             int t0 = 0;
 #pragma unroll 1
@@ -266,7 +275,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
                                 const uint32_t hi = t1 >= 32 ? 0xFFFFFFFFu : ((1u << t1) - 1u);
                                 const uint32_t msk = hi & ~((1u << t0) - 1u);
 #pragma unroll
-                                for (int t = 0; t < 32; ++t) acc = __fadd_rn(acc, ((msk >> t) & 1u) ? v[t] : 0.0f);
+                                for (int q = 0; q < 4; ++q) {
+                                    const uint32_t mq = (msk >> (8 * q)) & 0xFFu;
+                                    if (mq == 0) continue;
+#pragma unroll
+                                    for (int t = 0; t < 8; ++t)
+                                        acc = __fadd_rn(acc, ((mq >> t) & 1u) ? v[8 * q + t] : 0.0f);
+                                }
                                 if (t1 < cnt) {                // slice s ends at row col + t1
                                     if (hold) { held = acc; held_s = s; hold = false; }
                                     else if (o_bin >= 0) {
@@ -353,8 +368,7 @@ cudaError_t launch_front_tc_k(const FrontArgs &a, int per_sm, cudaStream_t s) {
     if (per_sm < 1) per_sm = 1;
     int grid = sms * per_sm;
     if (grid > a.n_events) grid = a.n_events;
-    k_front_tc<PREC, EDGE, NT><<<grid, NT, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_front_tc<PREC, EDGE, NT>, dim3(grid), dim3(NT), smem, s, a);
 }
 
 // CTAs per SM (the schedule's value): 1 or 2 run the two-warpgroup shape, 3 or 4 (and
