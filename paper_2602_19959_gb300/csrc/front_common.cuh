@@ -17,16 +17,12 @@ __device__ __forceinline__ int slice_of(float z) {
     return (int)floorf(q);
 }
 
-// Stores the 16 channels of storage row `row` of event e: channel-last float32 rows for
-// the FP32 form, plane-major rows (two 16-bit planes / one e4m3 plane) otherwise.
+// Stores the 16 channels of plane-major storage row `row` of event e (two 16-bit planes, one e4m3
+// plane).
 template <class T>
 __device__ __forceinline__ void store_row16(void *base, int64_t e, int64_t rows_e, int64_t row,
                                             const float v[kC0], float inv_scale) {
-    if constexpr (sizeof(T) == 4) {
-        float4 *d = reinterpret_cast<float4 *>(reinterpret_cast<float *>(base) + (e * rows_e + row) * kC0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-    } else if constexpr (sizeof(T) == 2) {
+    if constexpr (sizeof(T) == 2) {
         unsigned char *cb = reinterpret_cast<unsigned char *>(base);
         *reinterpret_cast<uint4 *>(cb + planar_off(e, 0, 2, rows_e, row)) = pack8<T>(v);
         *reinterpret_cast<uint4 *>(cb + planar_off(e, 1, 2, rows_e, row)) = pack8<T>(v + 8);
@@ -114,11 +110,14 @@ __device__ __forceinline__ int entry_slice(int en, const uint8_t *sslice) {
 // slice s whose slice-relative z (float32) is below a.edge also fills s - 1 (s > 0); one
 // at or above a.edge_hi = 10 - a.edge also fills s + 1 (s < 39).
 // EDGE = false: no boundary tracks (a.edge is 0). scnt/srun must hold 48 ints each.
+// SPLIT: an event shared by `nrank` blocks (a power of two), of which this one takes the slices
+// s = rank modulo nrank: the other slices come out empty.
 // Every thread of the block must call this.
-template <int NT, bool EDGE>
+template <int NT, bool EDGE, bool SPLIT = false>
 __device__ __forceinline__ void validate_sort(const FrontArgs &a, int ge, int tid, int *scnt, int *sseg,
                                               int *srun, uint16_t *ssorted, uint8_t *sslice,
-                                              int64_t &t0_out, int &nvalid_out) {
+                                              int64_t &t0_out, int &nvalid_out, int rank = 0, int nrank = 1) {
+    const auto own = [&](int s) { return !SPLIT || (s & (nrank - 1)) == rank; };
     const int src = a.ev_index ? a.ev_index[ge] : ge;      // gathered events: store index
     const int64_t t0 = a.offsets[src], t1 = a.offsets[src + 1];
     const bool bypass = t0 < 0 || t1 < t0 || t1 > a.n_tracks || (t1 - t0) > a.max_tracks;
@@ -139,12 +138,13 @@ __device__ __forceinline__ void validate_sort(const FrontArgs &a, int ge, int ti
         const int s = finite ? slice_of(z) : -1;
         int tag = 0;
         if (s >= 0) {
-            atomicAdd(&scnt[s], 1);
+            if (own(s)) atomicAdd(&scnt[s], 1);
             if constexpr (EDGE) {
                 const float zr = __fsub_rn(z, -100.0f + 10.0f * (float)s);   // as feature 2
                 if (s > 0 && zr < a.edge) tag = 1;
                 else if (s < kSlices - 1 && zr >= a.edge_hi) tag = 2;
-                if (tag) atomicAdd(&scnt[s - (tag & 1) + (tag >> 1)], 1);
+                const int s2 = s - (tag & 1) + (tag >> 1);
+                if (tag && own(s2)) atomicAdd(&scnt[s2], 1);
             }
         }
         sslice[t] = s < 0 ? 255 : (uint8_t)(s | (tag << 6));
@@ -185,6 +185,7 @@ __device__ __forceinline__ void validate_sort(const FrontArgs &a, int ge, int ti
                         en = t | (tag << 14);
                     }
                 }
+                if (!own(s)) s = 255;
                 const unsigned peers = __match_any_sync(0xffffffffu, s);
                 const unsigned lower = peers & ((1u << lane) - 1u);
                 int before = 0;
@@ -212,16 +213,12 @@ __device__ __forceinline__ void track_features(const FrontArgs &a, int64_t gt, i
     for (int k = kFeatures; k < kFcInPad; ++k) x[k] = 0.0f;
 }
 
-// Stores channels [8 h, 8 h + 8) of storage row `row` of event e: half a channel-last
-// float32 row, one of the two 16-bit planes, or half of the e4m3 plane's 16-byte row.
+// Stores channels [8 h, 8 h + 8) of storage row `row` of event e: one of the two 16-bit planes, or
+// half of the e4m3 plane's 16-byte row.
 template <class T>
 __device__ __forceinline__ void store_half8(void *base, int64_t e, int64_t rows_e, int64_t row, int h,
                                             const float v[8], float inv_scale) {
-    if constexpr (sizeof(T) == 4) {
-        float4 *d = reinterpret_cast<float4 *>(reinterpret_cast<float *>(base) + (e * rows_e + row) * kC0 + 8 * h);
-        d[0] = make_float4(v[0], v[1], v[2], v[3]);
-        d[1] = make_float4(v[4], v[5], v[6], v[7]);
-    } else if constexpr (sizeof(T) == 2) {
+    if constexpr (sizeof(T) == 2) {
         *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(base) + planar_off(e, h, 2, rows_e, row)) =
             pack8<T>(v);
     } else {
@@ -407,25 +404,14 @@ __device__ __forceinline__ void enc1_pool_quads(const FrontArgs &a, int e, int t
     }
 }
 
-// Channels [16 g, 16 g + 16) of storage row `row` of event e in a channel-last float32
-// tensor of C0 channels.
-template <int C0>
-__device__ __forceinline__ void store_seg16_f32(void *base, int64_t e, int64_t rows_e, int64_t row, int g,
-                                                const float v[16]) {
-    float4 *d = reinterpret_cast<float4 *>(reinterpret_cast<float *>(base) + (e * rows_e + row) * C0 + 16 * g);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-}
-
-// Step f with the weights read from shared memory per position pair, for the float32 front,
-// whose FC registers leave no room for them (same arithmetic, same order). senc holds
-// W[t][co] (5 C0 floats) then b[co]; the C0 channels are produced 16 at a time. A width
-// above 16 exists only in the float32 form.
+// Step f of the wide network's tensor-core forms, the weights read from shared memory per position
+// pair (same arithmetic, same order). senc holds W[t][co] (5 C0 floats) then b[co]; the C0 channels
+// are produced 16 at a time, two to a packed FMA.
 template <class T, int NT, bool AMAX, int C0>
 __device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, int tid, const float *shist,
                                                    const float *senc) {
-    static_assert(C0 % 16 == 0, "16-channel segments");
-    const int64_t rows1 = padded_rows(kBins), rows2 = padded_rows(kBins / 2);
+    static_assert(C0 % 16 == 0 && sizeof(T) <= 2, "16-channel segments, plane-major forms");
+    const int64_t rows2 = padded_rows(kBins / 2);
     const float inv = a.e1_inv_scale;
     float vmax = 0.0f;
     for (int q = tid; q < kBins / 2; q += NT) {
@@ -439,32 +425,27 @@ __device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, in
         for (int g = 0; g < C0 / 16; ++g) {
             float v0[16], v1[16], vp[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int co = 16 * g + j;
-                float a0 = senc[5 * C0 + co], a1 = a0;
+            for (int j = 0; j < 16; j += 2) {
+                const float *wj = senc + 16 * g + j;
+                float2 a0 = *reinterpret_cast<const float2 *>(wj + 5 * C0), a1 = a0;
 #pragma unroll
                 for (int t = 0; t < 5; ++t) {
-                    a0 = fmaf(senc[t * C0 + co], hv[t], a0);
-                    a1 = fmaf(senc[t * C0 + co], hv[t + 1], a1);
+                    const float2 w = *reinterpret_cast<const float2 *>(wj + t * C0);
+                    a0 = __ffma2_rn(w, make_float2(hv[t], hv[t]), a0);
+                    a1 = __ffma2_rn(w, make_float2(hv[t + 1], hv[t + 1]), a1);
                 }
-                v0[j] = leaky(a0);
-                v1[j] = leaky(a1);
-                vp[j] = fmaxf(v0[j], v1[j]);
-                if constexpr (AMAX) vmax = fmaxf(vmax, fmaxf(fabsf(v0[j]), fabsf(v1[j])));
+                a0 = leaky2(a0);
+                a1 = leaky2(a1);
+                v0[j] = a0.x; v0[j + 1] = a0.y;
+                v1[j] = a1.x; v1[j + 1] = a1.y;
+                vp[j] = fmaxf(a0.x, a1.x);
+                vp[j + 1] = fmaxf(a0.y, a1.y);
+                if constexpr (AMAX)
+                    vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(a0.x), fabsf(a1.x))), fmaxf(fabsf(a0.y), fabsf(a1.y)));
             }
-            if constexpr (C0 == kC0) {
-                store_row16<T>(a.e1, e, rows1, 2 * q + kPad, v0, inv);
-                store_row16<T>(a.e1, e, rows1, 2 * q + 1 + kPad, v1, inv);
-                store_row16<T>(a.p1, e, rows2, q + kPad, vp, inv);
-            } else if constexpr (sizeof(T) == 4) {
-                store_seg16_f32<C0>(a.e1, e, rows1, 2 * q + kPad, g, v0);
-                store_seg16_f32<C0>(a.e1, e, rows1, 2 * q + 1 + kPad, g, v1);
-                store_seg16_f32<C0>(a.p1, e, rows2, q + kPad, g, vp);
-            } else {   // the wide network in the tensor-core forms: plane-major segments
-                store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), 2 * q, g, v0, inv);
-                store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), 2 * q + 1, g, v1, inv);
-                store_seg16_pm<T, C0>(a.p1, e, rows2, q + kPad, g, vp, inv);
-            }
+            store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), 2 * q, g, v0, inv);
+            store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), 2 * q + 1, g, v1, inv);
+            store_seg16_pm<T, C0>(a.p1, e, rows2, q + kPad, g, vp, inv);
         }
     }
     if constexpr (AMAX) {
@@ -473,100 +454,83 @@ __device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, in
         if ((tid & 31) == 0) atomicMax(reinterpret_cast<int *>(a.amax), __float_as_int(vmax));
     }
     if (tid < 4) {
-        const int r = tid < 2 ? tid : kBins + tid;
-        const int rp = tid < 2 ? tid : kBins / 2 + tid;
-        if constexpr (C0 == kC0) {
-            zero_row16<T>(a.e1, e, rows1, r);
-            zero_row16<T>(a.p1, e, rows2, rp);
-        } else {
-            float z[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) z[i] = 0.0f;
-            for (int g = 0; g < C0 / 16; ++g) {
-                if constexpr (sizeof(T) == 4) {
-                    store_seg16_f32<C0>(a.e1, e, rows1, r, g, z);
-                    store_seg16_f32<C0>(a.p1, e, rows2, rp, g, z);
-                } else {
-                    store_seg16_quad<T, C0>(a.e1, e, quad_rows(kBins), r - kPad, g, z, 1.0f);
-                    store_seg16_pm<T, C0>(a.p1, e, rows2, rp, g, z, 1.0f);
-                }
-            }
-        }
+        const float z[16] = {};
+        zero_quad<T, C0>(a.e1, e, quad_rows(kBins), tid < 2 ? tid - kPad : kBins + tid - kPad);
+        for (int g = 0; g < C0 / 16; ++g)
+            store_seg16_pm<T, C0>(a.p1, e, rows2, tid < 2 ? tid : kBins / 2 + tid, g, z, 1.0f);
     }
 }
 
-// Step f in the per-interval layout (float32 form): e1 and p1 hold kSlices sequences per
-// event (sequence e * kSlices + s = interval s), each the conv of the interval's kIvLen-bin
-// window -- the interval's bins with kIvPad zero bins on each side -- with zero padding
-// beyond the window, as each interval runs the UNet on its own. Same arithmetic per
-// position as enc1_pool_shared_t.
-template <int NT, int C0>
-__device__ __forceinline__ void enc1_pool_windows_f32(const FrontArgs &a, int e, int tid, const float *shist,
-                                                      const float *senc) {
-    constexpr int Q = kIvLen / 2;                 // position pairs per window
-    const int64_t rows1 = padded_rows(kIvLen), rows2 = padded_rows(kIvLen / 2);
-    for (int idx = tid; idx < kSlices * Q; idx += NT) {
-        const int s = idx / Q, q = idx % Q;
-        const int64_t seq = (int64_t)e * kSlices + s;
+// Step f of the float32 form, channel-last rows, by `nt` threads (several blocks of an event where
+// they share it). Thread tid owns channels [4 h, 4 h + 4), h = tid modulo C0 / 4, of every position
+// pair it takes: its 20 weights and 4 biases stay in registers (read from shared memory per pair
+// they bound the step), and the threads of a pair write whole rows. Same arithmetic per position
+// as the other forms. IV: the per-interval layout, kSlices sequences per event (sequence
+// e * kSlices + s = interval s), each the conv of the interval's kIvLen-bin window -- the
+// interval's bins with kIvPad zero bins on each side -- with zero padding beyond the window, as
+// each interval runs the UNet on its own.
+template <int C0, bool IV>
+__device__ __forceinline__ void enc1_pool_f32(const FrontArgs &a, int e, int tid, int nt, const float *shist,
+                                              const float *senc) {
+    constexpr int H = C0 / 4, L = IV ? kIvLen : kBins, Q = L / 2, NS = IV ? kSlices : 1;
+    const int64_t rows1 = padded_rows(L), rows2 = padded_rows(Q);
+    const int h = tid % H;
+    float2 w[5][2], bias[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+#pragma unroll
+        for (int t = 0; t < 5; ++t) w[t][j] = *reinterpret_cast<const float2 *>(senc + t * C0 + 4 * h + 2 * j);
+        bias[j] = *reinterpret_cast<const float2 *>(senc + 5 * C0 + 4 * h + 2 * j);
+    }
+    float *e1 = reinterpret_cast<float *>(a.e1) + (int64_t)e * NS * rows1 * C0 + 4 * h;
+    float *p1 = reinterpret_cast<float *>(a.p1) + (int64_t)e * NS * rows2 * C0 + 4 * h;
+    for (int idx = tid / H; idx < NS * Q; idx += nt / H) {
+        const int s = IV ? idx / Q : 0, q = IV ? idx % Q : idx;
         float hv[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const int b = 2 * q + k - 2 - kIvPad;     // bin of the interval at window position 2q + k - 2
-            hv[k] = (b >= 0 && b < kSliceBins) ? shist[s * kSliceBins + b] : 0.0f;
+            const int b = 2 * q + k - 2 - (IV ? kIvPad : 0);      // bin of the event, or of the interval
+            hv[k] = (b >= 0 && b < (IV ? kSliceBins : kBins)) ? shist[s * kSliceBins + b] : 0.0f;
         }
-#pragma unroll 1
-        for (int g = 0; g < C0 / 16; ++g) {
-            float v0[16], v1[16], vp[16];
+        float4 v[2];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int co = 16 * g + j;
-                float a0 = senc[5 * C0 + co], a1 = a0;
+        for (int i = 0; i < 2; ++i) {
+            float2 acc[2] = {bias[0], bias[1]};
 #pragma unroll
-                for (int t = 0; t < 5; ++t) {
-                    a0 = fmaf(senc[t * C0 + co], hv[t], a0);
-                    a1 = fmaf(senc[t * C0 + co], hv[t + 1], a1);
-                }
-                v0[j] = leaky(a0);
-                v1[j] = leaky(a1);
-                vp[j] = fmaxf(v0[j], v1[j]);
-            }
-            store_seg16_f32<C0>(a.e1, seq, rows1, 2 * q + kPad, g, v0);
-            store_seg16_f32<C0>(a.e1, seq, rows1, 2 * q + 1 + kPad, g, v1);
-            store_seg16_f32<C0>(a.p1, seq, rows2, q + kPad, g, vp);
+            for (int t = 0; t < 5; ++t)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) acc[j] = __ffma2_rn(w[t][j], make_float2(hv[i + t], hv[i + t]), acc[j]);
+            acc[0] = leaky2(acc[0]);
+            acc[1] = leaky2(acc[1]);
+            v[i] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+            *reinterpret_cast<float4 *>(e1 + ((int64_t)s * rows1 + 2 * q + i + kPad) * C0) = v[i];
         }
+        *reinterpret_cast<float4 *>(p1 + ((int64_t)s * rows2 + q + kPad) * C0) =
+            make_float4(fmaxf(v[0].x, v[1].x), fmaxf(v[0].y, v[1].y), fmaxf(v[0].z, v[1].z), fmaxf(v[0].w, v[1].w));
     }
-    // the pad rows of every window: 0, 1 and L + 2, L + 3
-    float z[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) z[i] = 0.0f;
-    for (int idx = tid; idx < kSlices * 4; idx += NT) {
+    // the pad rows of every sequence: 0, 1 and L + 2, L + 3
+    const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int idx = tid / H; idx < NS * 4; idx += nt / H) {
         const int s = idx >> 2, k = idx & 3;
-        const int64_t seq = (int64_t)e * kSlices + s;
-        const int r = k < 2 ? k : kIvLen + k, rp = k < 2 ? k : kIvLen / 2 + k;
-        for (int g = 0; g < C0 / 16; ++g) {
-            store_seg16_f32<C0>(a.e1, seq, rows1, r, g, z);
-            store_seg16_f32<C0>(a.p1, seq, rows2, rp, g, z);
-        }
+        *reinterpret_cast<float4 *>(e1 + ((int64_t)s * rows1 + (k < 2 ? k : L + k)) * C0) = z;
+        *reinterpret_cast<float4 *>(p1 + ((int64_t)s * rows2 + (k < 2 ? k : Q + k)) * C0) = z;
     }
 }
 
-// REGW: weights in registers (tensor-core front, width 16) or read from shared memory
-// (float32 front, width C0).
-template <class T, int NT, bool REGW = true, int C0 = kC0, bool IV = false>
+// The tensor-core forms' step f: weights in registers at width 16 (IV: the per-interval layout),
+// read from shared memory at width 32.
+template <class T, int NT, int C0 = kC0, bool IV = false>
 __device__ __forceinline__ void enc1_pool(const FrontArgs &a, int e, int tid, const float *shist,
                                           const float *senc) {
-    if constexpr (REGW) {
-        static_assert(C0 == kC0, "register weights for width 16");
-        if constexpr (IV) {
-            if (a.amax) enc1_pool_t<T, NT, true>(a, e, tid, shist, senc);
-            else enc1_pool_t<T, NT, false>(a, e, tid, shist, senc);
-        } else {
-            if (a.amax) enc1_pool_quads<T, NT, true>(a, e, tid, shist, senc);
-            else enc1_pool_quads<T, NT, false>(a, e, tid, shist, senc);
-        }
-    } else {
+    if constexpr (C0 != kC0) {
         if (a.amax) enc1_pool_shared_t<T, NT, true, C0>(a, e, tid, shist, senc);
         else enc1_pool_shared_t<T, NT, false, C0>(a, e, tid, shist, senc);
+    } else if constexpr (IV) {
+        if (a.amax) enc1_pool_t<T, NT, true>(a, e, tid, shist, senc);
+        else enc1_pool_t<T, NT, false>(a, e, tid, shist, senc);
+    } else {
+        if (a.amax) enc1_pool_quads<T, NT, true>(a, e, tid, shist, senc);
+        else enc1_pool_quads<T, NT, false>(a, e, tid, shist, senc);
     }
 }
 

@@ -322,8 +322,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
             for (int i = tid; i < kBins / 4; i += kT) dst[i] = src[i];
         }
         if (!a.e1) {}                                    // the histogram alone was asked for
-        else if (a.iv) enc1_pool<T, kT, true, kC0, true>(a, e, tid, shist, senc);
-        else if (a.c0 == kC0Max) enc1_pool<T, kT, false, kC0Max>(a, e, tid, shist, senc);   // the wide network
+        else if (a.iv) enc1_pool<T, kT, kC0, true>(a, e, tid, shist, senc);
+        else if (a.c0 == kC0Max) enc1_pool<T, kT, kC0Max>(a, e, tid, shist, senc);   // the wide network
         else enc1_pool<T, kT>(a, e, tid, shist, senc);
         if (tid == 0) {
             int next = e + (int)gridDim.x;

@@ -140,13 +140,8 @@ void fill_f32(const std::vector<HostLayer> &Ls, const F32Layout &L, int c0, std:
     for (int l = 0; l < 6; ++l) {
         const HostLayer &H = Ls[l];
         const int nout = H.shape[0], nin = H.shape[1];
-        const int pitch = l == 0 ? kFcInPad : kFcHidden;
         for (int o = 0; o < nout; ++o)
-            for (int i = 0; i < nin; ++i) {
-                const float w = H.w[(size_t)o * nin + i];
-                if (l < 5) fc[fc_w_off(l) + o * pitch + i] = w;
-                else fc[fc_w_off(l) + i * kFcOut + o] = w;      // layer 6 transposed
-            }
+            for (int i = 0; i < nin; ++i) fc[fc_w_off(l) + i * nout + o] = H.w[(size_t)o * nin + i];
         for (int o = 0; o < nout; ++o) fc[fc_b_off(l) + o] = H.b[o];
     }
     {   // enc1 W[co][0][t] -> [t][co]

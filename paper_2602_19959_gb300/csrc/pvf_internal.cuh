@@ -43,8 +43,8 @@ constexpr float kThreshold = 0.01f;
 constexpr int kPeakHalfWin = 5;
 constexpr int kCentroidHalf = 3;
 
-// FC weights in float32. Layers 1-5: W[out][in] row-major, layer 1 padded to 12 inputs;
-// layer 6 transposed, W6T[in][out] (bin-parallel output layer); then all biases.
+// FC weights in float32, every layer transposed, W[in][out] (the float32 front reads the weights of
+// neighbouring outputs together), layer 1 padded to 12 inputs; then all biases.
 constexpr int kFcW1 = kFcHidden * kFcInPad;          // 384
 constexpr int kFcWH = kFcHidden * kFcHidden;         // 1024
 constexpr int kFcW6 = kFcOut * kFcHidden;            // 3200
