@@ -51,3 +51,22 @@ def test_tile_edges_and_shared_events(precision, tol, crowd, edge):
         assert np.array_equal(run(pick).view(np.int32), got[pick].view(np.int32)), m
     assert pv.device_status() == 0
     pv.close()
+
+
+def test_track_pointers_of_a_matrix_and_of_its_rows():
+    """The addresses taken from a matrix are those of its nine rows, in every form that is taken,
+    and what the rows are refused for the matrix is refused for."""
+    from paper_2602_19959_gb300.pvf import tracks_struct
+    m = torch.zeros((12, 64), device="cuda")
+    taken = [m, m[:9], m[1:], m[2:11, 3:40], m[:, :1], m[:, 5:5], m[::1, 7:8], m.int(), m[:1].expand(9, 64),
+             m[:, ::64], m.t().contiguous().t()[:, :1], torch.zeros((18, 8), device="cuda")[::2],
+             torch.zeros((9, 0), device="cuda"), torch.nn.Parameter(m), m.view(12, 64, 1), m.view(12, 8, 8), m[0]]
+    for t in taken:
+        a, b = tracks_struct(t), tracks_struct([t[k] for k in range(9)])
+        assert a.n_tracks == b.n_tracks and list(a.f) == list(b.f), tuple(t.shape)
+    refused = [m.t().contiguous().t(), m[:, ::2], m.half(), m.double(), m.cpu(), m[:8]]
+    for t in refused:
+        with pytest.raises((ValueError, IndexError)):
+            tracks_struct(t)
+        with pytest.raises((ValueError, IndexError)):
+            tracks_struct([t[k] for k in range(9)])
