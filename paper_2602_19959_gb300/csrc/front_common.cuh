@@ -237,10 +237,9 @@ __device__ __forceinline__ void store_half8(void *base, int64_t e, int64_t rows_
 // sequences end to end, each the conv of the interval's kIvLen-bin window (its bins with
 // kIvPad zero bins on each side), two zero rows before each sequence and two after the
 // last (neighbouring sequences share the two between them).
-template <class T, int NT, bool AMAX>
-__device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, const float *shist,
+template <class T, bool AMAX>
+__device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, int nt, const float *shist,
                                             const float *senc) {
-    static_assert(NT % 2 == 0, "thread pairs");
     constexpr int S1 = kIvLen + kPad, S2 = kIvLen / 2 + kPad;   // rows per sequence
     constexpr int RQ = quad_rows(kSlices * S1 - kPad);     // e1: the quad layout
     constexpr int64_t rows2 = (int64_t)kSlices * S2 + kPad;
@@ -256,7 +255,7 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
     }
     float vmax = 0.0f;
 #pragma unroll 2   // two position pairs in flight per thread: front 81.6 -> 79.5 us (FP16)
-    for (int qi = tid >> 1; qi < NQ; qi += NT / 2) {
+    for (int qi = tid >> 1; qi < NQ; qi += nt / 2) {
         // the pair's sequence and first position; e1 positions p1, p1 + 1, p1 row r2
         const int sq = qi / (kIvLen / 2), q = qi % (kIvLen / 2);
         const int p1 = sq * S1 + 2 * q;
@@ -315,7 +314,7 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
         for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
         if ((tid & 31) == 0) atomicMax(reinterpret_cast<int *>(a.amax), __float_as_int(vmax));
     }
-    for (int idx = tid; idx < (kSlices + 1) * 2; idx += NT) {   // the two rows before each sequence and after the last
+    for (int idx = tid; idx < (kSlices + 1) * 2; idx += nt) {   // the two rows before each sequence and after the last
         const int sq = idx >> 1, k = idx & 1;
         zero_quad<T, kC0>(a.e1, e, RQ, sq * S1 + k - kPad);
         zero_row16<T>(a.p1, e, rows2, (int64_t)sq * S2 + k);
@@ -326,8 +325,8 @@ __device__ __forceinline__ void enc1_pool_t(const FrontArgs &a, int e, int tid, 
 // eight histogram bins (shist is zero for two bins on either side), their addresses (one row of
 // the four residue planes of e1, two rows of p1) and, in registers, the weights of the thread's 8
 // channels. Same arithmetic per position as enc1_pool_t.
-template <class T, int NT, bool AMAX>
-__device__ __forceinline__ void enc1_pool_quads(const FrontArgs &a, int e, int tid, const float *shist,
+template <class T, bool AMAX>
+__device__ __forceinline__ void enc1_pool_quads(const FrontArgs &a, int e, int tid, int nt, const float *shist,
                                                 const float *senc) {
     static_assert(sizeof(T) <= 2 && kBins % 4 == 0, "plane-major forms");
     constexpr int RQ = quad_rows(kBins);
@@ -347,7 +346,7 @@ __device__ __forceinline__ void enc1_pool_quads(const FrontArgs &a, int e, int t
     unsigned char *e1 = reinterpret_cast<unsigned char *>(a.e1) + quad_off(e, P == 2 ? h : 0, P, RQ, 0) + half * h;
     unsigned char *p1 = reinterpret_cast<unsigned char *>(a.p1) + planar_off(e, P == 2 ? h : 0, P, rows2, kPad) + half * h;
 #pragma unroll 1
-    for (int q = tid >> 1; q < kBins / 4; q += NT / 2) {
+    for (int q = tid >> 1; q < kBins / 4; q += nt / 2) {
         float hv[8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -407,14 +406,14 @@ __device__ __forceinline__ void enc1_pool_quads(const FrontArgs &a, int e, int t
 // Step f of the wide network's tensor-core forms, the weights read from shared memory per position
 // pair (same arithmetic, same order). senc holds W[t][co] (5 C0 floats) then b[co]; the C0 channels
 // are produced 16 at a time, two to a packed FMA.
-template <class T, int NT, bool AMAX, int C0>
-__device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, int tid, const float *shist,
+template <class T, bool AMAX, int C0>
+__device__ __forceinline__ void enc1_pool_shared_t(const FrontArgs &a, int e, int tid, int nt, const float *shist,
                                                    const float *senc) {
     static_assert(C0 % 16 == 0 && sizeof(T) <= 2, "16-channel segments, plane-major forms");
     const int64_t rows2 = padded_rows(kBins / 2);
     const float inv = a.e1_inv_scale;
     float vmax = 0.0f;
-    for (int q = tid; q < kBins / 2; q += NT) {
+    for (int q = tid; q < kBins / 2; q += nt) {
         float hv[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -517,20 +516,20 @@ __device__ __forceinline__ void enc1_pool_f32(const FrontArgs &a, int e, int tid
     }
 }
 
-// The tensor-core forms' step f: weights in registers at width 16 (IV: the per-interval layout),
+// The tensor-core forms' step f by `nt` threads (of one block, or of those that share the event): weights in registers at width 16 (IV: the per-interval layout),
 // read from shared memory at width 32.
-template <class T, int NT, int C0 = kC0, bool IV = false>
-__device__ __forceinline__ void enc1_pool(const FrontArgs &a, int e, int tid, const float *shist,
+template <class T, int C0 = kC0, bool IV = false>
+__device__ __forceinline__ void enc1_pool(const FrontArgs &a, int e, int tid, int nt, const float *shist,
                                           const float *senc) {
     if constexpr (C0 != kC0) {
-        if (a.amax) enc1_pool_shared_t<T, NT, true, C0>(a, e, tid, shist, senc);
-        else enc1_pool_shared_t<T, NT, false, C0>(a, e, tid, shist, senc);
+        if (a.amax) enc1_pool_shared_t<T, true, C0>(a, e, tid, nt, shist, senc);
+        else enc1_pool_shared_t<T, false, C0>(a, e, tid, nt, shist, senc);
     } else if constexpr (IV) {
-        if (a.amax) enc1_pool_t<T, NT, true>(a, e, tid, shist, senc);
-        else enc1_pool_t<T, NT, false>(a, e, tid, shist, senc);
+        if (a.amax) enc1_pool_t<T, true>(a, e, tid, nt, shist, senc);
+        else enc1_pool_t<T, false>(a, e, tid, nt, shist, senc);
     } else {
-        if (a.amax) enc1_pool_quads<T, NT, true>(a, e, tid, shist, senc);
-        else enc1_pool_quads<T, NT, false>(a, e, tid, shist, senc);
+        if (a.amax) enc1_pool_quads<T, true>(a, e, tid, nt, shist, senc);
+        else enc1_pool_quads<T, false>(a, e, tid, nt, shist, senc);
     }
 }
 

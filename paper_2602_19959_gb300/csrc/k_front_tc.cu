@@ -23,6 +23,15 @@
 // order that depends only on the event's own sorted track list, so results are identical
 // alone, in any batch and under either shape. One thread issues the MMAs; every wait on
 // their completion is bounded.
+//
+// What bounds it: at 1000 events (76 us, 78 before enc1 took four positions per step and warps
+// without tracks left the hidden layers) the stores of e1 and p1, the softplus (two
+// special-function operations per track and lane) and the latency of six dependent MMAs per pass,
+// with four CTAs per SM to fill each other's gaps. Of one event's 33000 cycles enc1 took 9500 and
+// the output layer 9700: a launch with SMs to spare gives each event up to eight blocks, all of
+// which make the histogram (no exchange, and the sums keep their order) while each writes its
+// share of e1 and p1. One event 18 -> 13.5 us; a call 44.3 -> 40.5 (four blocks 41.0, sixteen the
+// same as eight).
 #include "front_common.cuh"
 #include "tc_ptx.cuh"
 
@@ -33,6 +42,7 @@ using namespace front;
 using namespace tc;
 
 constexpr int kRows = 128;              // tile rows = TMEM lanes
+constexpr int kMaxShare = 8;            // blocks that may share an event's enc1
 
 // NT threads = NT / 128 warpgroups, one 128-row tile each; a pass holds NT tracks.
 // TMEM: NT columns (hidden layers: tile g at column 128 g; output layer: [0, N)).
@@ -156,7 +166,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
     // persistent: the CTA walks the launch's events, its first one blockIdx.x, then the
     // next unclaimed one (a global ticket: CTAs that finish early take more events, and
     // each event is still computed whole by one CTA, so results do not depend on which)
-    for (int e = blockIdx.x; e < n_ev;) {
+    // a.share > 1 blocks per event, one event each: all make its histogram, and each writes its share
+    // of what follows
+    const int gtid = tid + kT * (int)(blockIdx.x & (unsigned)(a.share - 1)), nt = kT * a.share;
+    for (int e = (int)(blockIdx.x / (unsigned)a.share); e < n_ev;) {
         const int ge = a.ev_base + e;
         if (a.hist_in) {
             const float *src = a.hist_in + (size_t)ge * kBins;
@@ -319,15 +332,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_front_tc(FrontArgs a) {
         if (a.hist_out) {
             float4 *dst = reinterpret_cast<float4 *>(a.hist_out + (size_t)ge * kBins);
             const float4 *src = reinterpret_cast<const float4 *>(shist);
-            for (int i = tid; i < kBins / 4; i += kT) dst[i] = src[i];
+            for (int i = gtid; i < kBins / 4; i += nt) dst[i] = src[i];
         }
         if (!a.e1) {}                                    // the histogram alone was asked for
-        else if (a.iv) enc1_pool<T, kT, kC0, true>(a, e, tid, shist, senc);
-        else if (a.c0 == kC0Max) enc1_pool<T, kT, kC0Max>(a, e, tid, shist, senc);   // the wide network
-        else enc1_pool<T, kT>(a, e, tid, shist, senc);
+        else if (a.iv) enc1_pool<T, kC0, true>(a, e, gtid, nt, shist, senc);
+        else if (a.c0 == kC0Max) enc1_pool<T, kC0Max>(a, e, gtid, nt, shist, senc);   // the wide network
+        else enc1_pool<T>(a, e, gtid, nt, shist, senc);
         if (tid == 0) {
-            int next = e + (int)gridDim.x;
-            if (a.ev_ctr) {
+            int next = a.share > 1 ? n_ev : e + (int)gridDim.x;
+            if (a.ev_ctr && a.share == 1) {
                 // one ticket per processed event: the ticket n_ev - 1 is the launch's last,
                 // and its taker resets the counter for the next launch (CTAs without an
                 // event never touch it)
@@ -368,7 +381,13 @@ cudaError_t launch_front_tc_k(const FrontArgs &a, int per_sm, cudaStream_t s) {
     if (per_sm < 1) per_sm = 1;
     int grid = sms * per_sm;
     if (grid > a.n_events) grid = a.n_events;
-    return launch_pdl(k_front_tc<PREC, EDGE, NT>, dim3(grid), dim3(NT), smem, s, a);
+    // blocks that share an event's enc1: only on SMs that would be idle, so that no block making a
+    // histogram a second time slows another (nothing to share when the histogram alone is wanted)
+    FrontArgs b = a;
+    b.share = 1;
+    while (a.e1 && b.share < kMaxShare && 2 * b.share * (int64_t)a.n_events <= sms) b.share *= 2;
+    if (b.share > 1) grid = b.share * a.n_events;
+    return launch_pdl(k_front_tc<PREC, EDGE, NT>, dim3(grid), dim3(NT), smem, s, b);
 }
 
 // CTAs per SM (the schedule's value): 1 or 2 run the two-warpgroup shape, 3 or 4 (and
