@@ -176,6 +176,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_front(FrontArgs a) {
         for (int i = tid; i < kFcFloats / 4; i += kThreads)
             cp_async16(sfc + 4 * i, a.fc + 4 * i);     // arrive behind the first event's sort
 
+    // the caller's inputs, and the buffers that earlier calls' kernels may still read, only after the
+    // previous kernel of the stream has finished (no early trigger: see the launches of k_unet_f32.cu)
+    grid_dep_wait();
+
     // persistent: the CTA walks the launch's events (weights loaded once above)
     for (int e = blockIdx.x / nr; e < a.n_events; e += gridDim.x / nr) {
         const int ge = a.ev_base + e;
@@ -291,16 +295,25 @@ cudaError_t launch_front_t(const FrontArgs &a, size_t smem, cudaStream_t s) {
     int split = 1;
     while (split < kMaxSplit && 2 * split * (int64_t)a.n_events <= sms * per_sm) split *= 2;
     const int64_t most = split > 1 ? (int64_t)split * a.n_events : sms * per_sm;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim = {(unsigned)split, 1, 1};
+    // dependent launch as in launch_pdl, but not for the histogram alone, whose weights are copied to
+    // the static scratch by the call itself
+    cudaLaunchAttribute attr[2];
+    int n_attr = 0;
+    if (ENC1) {
+        attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (split > 1) {
+        attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+        attr[n_attr++].val.clusterDim = {(unsigned)split, 1, 1};
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(most < (int64_t)split * a.n_events ? most : (int64_t)split * a.n_events));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = split > 1 ? 1 : 0;
+    cfg.numAttrs = n_attr;
     return cudaLaunchKernelEx(&cfg, k_front<ENC1, EDGE, C0, IV>, a);
 }
 

@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(kThreads, CONV ? 2 : 4) k_tail(TailArgs a) {
         __syncthreads();
     }
     // the logits (or d1) are the previous kernel's output (dependent launch)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    grid_dep_wait();
+    grid_dep_launch();
     // persistent: the CTA walks the launch's events
     const int n_ev = launch_events(a.n_dyn, a.ev_base, a.n_events);
     // the logits of event e into buffer f (asynchronous copies)
@@ -246,9 +246,7 @@ cudaError_t launch_tail_t(const TailArgs &a, cudaStream_t s) {
     int per_sm = CONV ? 2 : 4;
     if (a.ctas_per_sm > 0 && a.ctas_per_sm < per_sm) per_sm = a.ctas_per_sm;
     const dim3 grid(a.n_events < per_sm * sms ? a.n_events : per_sm * sms), block(kThreads);
-    if (!CONV) return launch_pdl(k_tail<CONV, C0, IV>, grid, block, smem, s, a);
-    k_tail<CONV, C0, IV><<<grid, block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_tail<CONV, C0, IV>, grid, block, smem, s, a);
 }
 
 }  // namespace

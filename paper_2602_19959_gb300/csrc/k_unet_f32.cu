@@ -78,7 +78,7 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
     const int p0 = blockIdx.x * TP;
     const int64_t rowsE = padded_rows(L);
 
-    auto stage = [&](int kc, int buf) {
+    auto stage_x = [&](int kc, int buf) {
         const bool fromA = kc < CA;
         const int C = fromA ? CA : CB;
         const float *src = (fromA ? inA : inB) + (fromA ? kc : kc - CA);
@@ -90,6 +90,8 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
             const bool ok = srow < rowsE;
             cp4(&xs[buf][k][rr], src + ((e0 + s) * rowsE + (ok ? srow : 0)) * C + k, ok);
         }
+    };
+    auto stage_w = [&](int kc, int buf) {
         for (int idx = tid; idx < 5 * KC * COUT / 4; idx += NT) {
             const int t = idx / (KC * COUT / 4), rem = idx % (KC * COUT / 4);
             cp16(reinterpret_cast<float4 *>(&ws[buf][t][0][0]) + rem,
@@ -97,7 +99,7 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
         }
     };
 
-    stage(0, 0);
+    stage_w(0, 0);      // the handle's, like the biases; the inputs are the previous kernel's output
     float2 acc[8][4];                        // [position][channel pair]
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -106,13 +108,18 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
         for (int pi = 0; pi < 8; ++pi) acc[pi][q] = b;
     }
 
+    grid_dep_wait();
+    stage_x(0, 0);
     constexpr int NCH = CIN / KC;
 #pragma unroll 1
     for (int c = 0; c < NCH; ++c) {
         const int buf = c & 1;
         cp_wait_all();
         __syncthreads();                     // chunk c staged; the other buffer is no longer read
-        if (c + 1 < NCH) stage((c + 1) * KC, buf ^ 1);
+        if (c + 1 < NCH) {
+            stage_x((c + 1) * KC, buf ^ 1);
+            stage_w((c + 1) * KC, buf ^ 1);
+        }
 #pragma unroll 4   // against 1: dec3 664 -> 652, dec2 350 -> 339, enc2 107 -> 100 us (500 events)
         for (int k = 0; k < KC; ++k) {
             float xv[12];
@@ -212,7 +219,7 @@ k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
     const int Lout = 2 * Lin;
     const int64_t rowsOut = padded_rows(Lout);
 
-    auto stage = [&](int kc, int buf) {
+    auto stage_x = [&](int kc, int buf) {
         // 8 channels at a time: 32 contiguous bytes per position, distinct banks per warp
         for (int idx = tid; idx < NS * TP * KC; idx += NT) {
             const int k = idx % 8 + idx / (8 * NS * TP) * 8, rr = idx / 8 % (NS * TP);
@@ -220,12 +227,14 @@ k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
             const bool ok = p < Lin;
             cp4(&xs[buf][k][rr], in + ((e0 + s) * rowsIn + (ok ? p + kPad : 0)) * CIN + kc + k, ok);
         }
+    };
+    auto stage_w = [&](int kc, int buf) {
         for (int idx = tid; idx < KC * N / 4; idx += NT)
             cp16(reinterpret_cast<float4 *>(&ws[buf][0][0]) + idx,
                  reinterpret_cast<const float4 *>(W + (size_t)kc * N) + idx);
     };
 
-    stage(0, 0);
+    stage_w(0, 0);      // the handle's, like the biases; the inputs are the previous kernel's output
     float2 acc[8][8];                        // [position][column pair]
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
@@ -237,13 +246,18 @@ k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
             for (int pi = 0; pi < 8; ++pi) acc[pi][2 * g + h] = b;
         }
     }
+    grid_dep_wait();
+    stage_x(0, 0);
     constexpr int NCH = CIN / KC;
 #pragma unroll 1
     for (int c = 0; c < NCH; ++c) {
         const int buf = c & 1;
         cp_wait_all();
         __syncthreads();
-        if (c + 1 < NCH) stage((c + 1) * KC, buf ^ 1);
+        if (c + 1 < NCH) {
+            stage_x((c + 1) * KC, buf ^ 1);
+            stage_w((c + 1) * KC, buf ^ 1);
+        }
 #pragma unroll 2
         for (int k = 0; k < KC; ++k) {
             const float4 *xr = reinterpret_cast<const float4 *>(&xs[buf][k][sq * TP + pg * 8]);
@@ -288,22 +302,26 @@ k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
     }
 }
 
+// Dependent launches hide each other's launch and first weight tile. The kernels trigger nothing
+// early: blocks of the next layer placed while this one still ran crowded the SMs that happened to
+// be free (16 events: 184 us a call without dependent launches, 158 with them, 210 with a trigger
+// behind the main loop, 234 at the start; 500 events 2333, 2312, 2312, 2366).
+
 // n: sequences (a multiple of NS)
 template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC>
 cudaError_t conv5(const void *a, const void *b, const float *W, const float *bias, void *out,
                   void *outp, int L, int n, cudaStream_t s) {
     dim3 grid((L + TP - 1) / TP, n / NS), block((TP / 8) * (COUT / 8) * NS);
-    k_conv5_f32<CA, CB, COUT, TP, NS, POOL, KC><<<grid, block, 0, s>>>(
-        (const float *)a, (const float *)b, W, bias, (float *)out, (float *)outp, L);
-    return cudaGetLastError();
+    return launch_pdl(k_conv5_f32<CA, CB, COUT, TP, NS, POOL, KC>, grid, block, 0, s, (const float *)a,
+                      (const float *)b, W, bias, (float *)out, (float *)outp, L);
 }
 
 template <int CIN, int COUT, int TP, int NS, int KC>
 cudaError_t convT(const void *in, const float *W, const float *bias, void *out, int Lin, int n,
                   cudaStream_t s) {
     dim3 grid((Lin + TP - 1) / TP, n / NS), block((TP / 8) * (2 * COUT / 16) * NS);
-    k_convT_f32<CIN, COUT, TP, NS, KC><<<grid, block, 0, s>>>((const float *)in, W, bias, (float *)out, Lin);
-    return cudaGetLastError();
+    return launch_pdl(k_convT_f32<CIN, COUT, TP, NS, KC>, grid, block, 0, s, (const float *)in, W, bias,
+                      (float *)out, Lin);
 }
 
 // The layer sequence for base width C (levels C, 2C, 4C, 8C). Tiles halve as the channel

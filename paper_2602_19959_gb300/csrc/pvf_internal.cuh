@@ -318,6 +318,13 @@ struct ProfScope {
     ~ProfScope() { if (h) h->end(h->ctx, s); }
 };
 
+// Programmatic dependent launch (kernels launched with the programmatic stream
+// serialization attribute): wait until the previous kernel in the stream has completed
+// and its writes are visible; then allow the next kernel to launch. Both are no-ops for
+// a kernel launched without the attribute.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Launch with programmatic stream serialization: the kernel may start while the previous
 // kernel of the stream finishes; it must call griddepcontrol.wait before reading that
 // kernel's output, and triggers its own dependents only after that wait, so at most two
