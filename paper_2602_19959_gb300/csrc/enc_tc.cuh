@@ -33,7 +33,7 @@ template <class N> struct Enc {
     using C4 = typename N::Enc4Up3;
     static constexpr int T2N = C2::TPE, T3N = C3::TPE, T4N = C4::TPE;    // tiles per event
     static_assert(T2N == 2 * T3N && T3N == 2 * T4N && T4N % 4 == 0, "4 : 2 : 1 tiles");
-    static_assert(C2::L == 2 * C3::L && C3::L == 2 * C4::L && C4::A2T && !C2::SEQ, "whole events");
+    static_assert(C2::L == 2 * C3::L && C3::L == 2 * C4::L && !C2::SEQ, "whole events");
     static constexpr int ST = 3;                    // p1 stages
     static constexpr int NP2 = 3, NP3 = 3;          // p2 / p3 operand tiles
     static constexpr int RING = 8;                  // tile-done barriers of enc2 and enc3

@@ -5,27 +5,29 @@
 // here they are the BF16, FP16 and FP8 (E4M3) forms.
 //
 // Kernel families (each a persistent, warp-specialised kernel):
-//   enc2      conv 16->32  @2000, epilogue also writes the 2:1 max-pool
-//   enc3      conv 32->64  @1000, + pool
-//   enc4_up3  conv 64->128 @500,  epilogue feeds a second GEMM: ConvT 128->64 (k2 s2)
+//   enc_up3   convs 16->32 @2000 + pool, 32->64 @1000 + pool, 64->128 @500 + ConvT 128->64 (k2 s2)
+//             of whole events at base width 16, as one kernel: enc_tc.cuh
+//   enc2, enc3, enc4_up3   the same layers one by one, for the per-interval layout
 //   dec3_up2  conv [64|64]->64 @1000, + ConvT 64->32
 //   dec2_up1  conv [32|32]->32 @2000, + ConvT 32->16
 //   dec1      conv [16|16]->16 @4000, + the final conv 16->1 (logits): dec1_tc.cuh
+// and the wide network's (enc2, enc3, enc4, up3, dec3, up2, dec2_up1, dec1).
 // The skip concat is never materialised: the two inputs are copied into adjacent
 // K-planes of the same shared-memory tile. Every conv and ConvT output goes through
-// LeakyReLU(0.01) in the epilogue; the fused ConvT reads the conv tile from shared
-// memory, so the deepest level's activations (e4, d3, d2) never reach global memory.
+// LeakyReLU(0.01) in the epilogue; a fused ConvT reads the conv tile from tensor memory, where
+// the epilogue puts it in the storage type, so those activations (e4, d3, d2) never reach
+// global memory. Biases and column scales are launch parameters (constant cache): read from
+// shared memory they took four cycles of its data path per 16 bytes and warp.
 //
 // Warp roles: warp 0 issues the bulk copies (weights once, then one halo'd activation
 // tile per 128 positions into a ring of stages); warp 1 allocates TMEM and one thread
 // issues the MMAs into NB accumulator buffers, so the MMAs of tile i wait only for the
 // epilogue of tile i - NB; the remaining one, two or four warpgroups are the epilogue,
-// one TMEM lane (= output position) per thread. With a fused ConvT and two or four
-// epilogue warpgroups they split by role: half of them turn each conv accumulator into
-// the ConvT's shared-memory operand, the other half store the ConvT output (written over
-// the conv columns, already read) and free the buffer, so the operand of tile i is ready
-// while the tensor core still runs the conv of tile i + 1; the two warpgroups of a role
-// (if four) split its columns. Otherwise two warpgroups split the accumulator columns.
+// one TMEM lane (= output position) per thread. With a fused ConvT they split by role: half
+// of them turn each conv accumulator into the ConvT's operand, the other half store the ConvT
+// output (written over the conv columns, already read) and free the buffer, so the operand of
+// tile i is ready while the tensor core still runs the conv of tile i + 1; the two warpgroups
+// of a role (if four) split its columns. Otherwise two warpgroups split the accumulator columns.
 //
 // Tap pairing (the 16-bit forms' dec3_up2 and dec2_up1): a tcgen05.mma costs about the same for
 // N up to 64 (reading A dominates), so the small-C_out convs stack two taps' weights in N:
@@ -74,7 +76,7 @@ __host__ __device__ constexpr int pow2ceil(int x) {
 __host__ __device__ constexpr int align_up(int x, int a) { return (x + a - 1) / a * a; }
 
 template <int PREC_, int CA_, int CB_, int COUT_, int L_, int EPI_, int CUP_, int STAGES_, int EWG_ = 1,
-          int MAXREG_ = 128, int NB_ = 2, bool PAIRED_ = false, bool DYN_ = false, bool A2T_ = false,
+          int MAXREG_ = 128, int NB_ = 2, bool PAIRED_ = false, bool DYN_ = false,
           int SEQ_ = 0, int NSPLIT_ = 1>
 struct Cfg {
     static constexpr int PREC = PREC_;
@@ -135,12 +137,10 @@ struct Cfg {
     static constexpr int N2 = EPI == EPI_UP ? 2 * CUP : 0;   // fused ConvT: n = r * CUP + co
     static constexpr int P2 = COUT / PW;                     // K-planes of the fused GEMM
     static constexpr int W2_BYTES = EPI == EPI_UP ? P2 * N2 * 16 : 0;
-    // the fused ConvT's A operand (the conv output of the tile, quantised): in shared memory,
-    // or (A2T) in tensor memory, written by the epilogue with tcgen05.st and read by the
-    // MMA directly, which takes its traffic off the shared-memory pipe
-    static constexpr bool A2T = A2T_ && EPI == EPI_UP;
-    static constexpr int A2_BYTES = EPI == EPI_UP && !A2T ? P2 * kTileM * 16 : 0;
-    static constexpr int A2_COLS = A2T ? P2 * 4 : 0;         // a 16-byte plane row = 4 columns
+    // the fused ConvT's A operand (the conv output of the tile, quantised) in tensor memory, written
+    // by the epilogue with tcgen05.st and read by the MMA directly, which keeps its traffic off the
+    // shared-memory pipe
+    static constexpr int A2_COLS = EPI == EPI_UP ? P2 * 4 : 0;      // a 16-byte plane row = 4 columns
     // accumulator buffer: the fused ConvT writes its result over the conv columns, which
     // the epilogue has read before the ConvT's operand is complete
     static constexpr int CONV_COLS = PAIRED ? 2 * COUT : COUT;      // E | O when paired
@@ -155,9 +155,8 @@ struct Cfg {
     static constexpr int OFF_W = 0;
     static constexpr int OFF_W2 = align_up(OFF_W + W_BYTES, 128);
     static constexpr int OFF_A = align_up(OFF_W2 + W2_BYTES, 128);
-    static constexpr int OFF_A2 = OFF_A + STAGES * A_STAGE;
     // paired: each lane quarter's first O row, for the quarter above (two buffers)
-    static constexpr int OFF_X = align_up(OFF_A2 + 2 * A2_BYTES, 128);
+    static constexpr int OFF_X = align_up(OFF_A + STAGES * A_STAGE, 128);
     static constexpr int X_BYTES = PAIRED ? 2 * 4 * COUT * 4 : 0;
     static constexpr int OFF_BAR = align_up(OFF_X + X_BYTES, 128);
     static constexpr int SMEM = OFF_BAR + 512;
@@ -186,6 +185,7 @@ struct Cfg {
     static_assert(!SEQ || (L == kSlices * SEQ - kPad &&
                            (EPI != EPI_POOL || (SEQ % 2 == 0 && LSEQ % 2 == 0))),
                   "per-interval geometry");
+    static_assert(EPI != EPI_UP || EWG == 2 || EWG == 4, "the fused ConvT's two roles");
     static_assert(EPI != EPI_UP || CUP % 16 == 0, "16-column epilogue chunks");
     static_assert(EWG == 1 || (EWG == 2 && EPI_COLS % 16 == 0) ||
                   (EWG == 4 && EPI == EPI_UP && (COUT / 2) % 16 == 0 && (N2 / 2) % 16 == 0),
@@ -406,15 +406,7 @@ __device__ __forceinline__ void issue_conv(uint32_t d, uint32_t as, uint32_t w_b
     }
 }
 
-template <class C>
-__device__ __forceinline__ void issue_up(uint32_t d2, uint32_t a2, uint32_t w2_base) {
-    const uint64_t a0 = smem_desc(a2, kTileM * 16, 128), b0 = smem_desc(w2_base, C::N2 * 16, 128);
-#pragma unroll
-    for (int kb = 0; kb < C::P2 / 2; ++kb)
-        mma_t<C>(d2, desc_plus(a0, 2 * kb * kTileM), desc_plus(b0, 2 * kb * C::N2), C::IDESC2, kb != 0);
-}
-
-// The fused ConvT with its A operand in tensor memory (A2T): the K step kb reads the 8
+// The fused ConvT, its A operand in tensor memory: the K step kb reads the 8
 // columns holding channels [16 kb, 16 kb + 16) (16-bit; 32 e4m3 channels per step).
 template <class C>
 __device__ __forceinline__ void issue_up_ts(uint32_t d2, uint32_t a2_tmem, uint32_t w2_base) {
@@ -428,11 +420,8 @@ __device__ __forceinline__ void issue_up_ts(uint32_t d2, uint32_t a2_tmem, uint3
 }
 
 template <class C>
-__device__ __forceinline__ void issue_up_any(uint32_t tmem, int bp, int ap, uint32_t a2_base, uint32_t w2_base) {
-    if constexpr (C::A2T)
-        issue_up_ts<C>(tmem + bp * C::COLS_BUF + C::UP_OFF, tmem + C::A2_COL0 + ap * C::A2_COLS, w2_base);
-    else
-        issue_up<C>(tmem + bp * C::COLS_BUF + C::UP_OFF, a2_base + ap * C::A2_BYTES, w2_base);
+__device__ __forceinline__ void issue_up_any(uint32_t tmem, int bp, int ap, uint32_t w2_base) {
+    issue_up_ts<C>(tmem + bp * C::COLS_BUF + C::UP_OFF, tmem + C::A2_COL0 + ap * C::A2_COLS, w2_base);
 }
 
 // One thread issues all MMAs. With a fused ConvT,
@@ -451,7 +440,6 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
     const uint32_t a_base = smem_u32(smem + C::OFF_A);
     const uint32_t w_base = smem_u32(smem + C::OFF_W);
     const uint32_t w2_base = smem_u32(smem + C::OFF_W2);
-    const uint32_t a2_base = smem_u32(smem + C::OFF_A2);
     const int ntiles = a.n_events * C::TPE, step = (int)gridDim.x / C::NSPLIT;
     int s = 0, b = 0, bp = 0, r = 0;          // stage, accumulator, the previous tile's, ring slot
     uint32_t ph_s = 0, ph_b = 0, ph_r = 0;    // their parities
@@ -476,7 +464,7 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
                 const int ap = (i - 1) & 1;
                 if (!mbar_wait(&a2full[ap], ((i - 1) >> 1) & 1, abort)) { ok = false; break; }
                 tc_fence_after();
-                issue_up_any<C>(tmem, bp, ap, a2_base, w2_base);
+                issue_up_any<C>(tmem, bp, ap, w2_base);
                 mma_commit(&t2full[bp]);
             }
             bp = b;
@@ -489,7 +477,7 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
             const int ap = (i - 1) & 1;
             if (mbar_wait(&a2full[ap], ((i - 1) >> 1) & 1, abort)) {
                 tc_fence_after();
-                issue_up_any<C>(tmem, bp, ap, a2_base, w2_base);
+                issue_up_any<C>(tmem, bp, ap, w2_base);
                 mma_commit(&t2full[bp]);
             } else {
                 ok = false;
@@ -616,7 +604,7 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
                     for (int j = 0; j < 16; ++j) v[j] = 0.0f;
                 }
             }
-            if constexpr (C::EPI == EPI_UP && C::A2T) {
+            if constexpr (C::EPI == EPI_UP) {
                 // this row's 16 channels into its TMEM lane: 16-bit pairs (8 columns) or
                 // e4m3 quads (4 columns), the K order the MMA reads
                 if constexpr (CAL) amax_fold(a.amax, a.amax_mid, v, valid);
@@ -631,10 +619,6 @@ __device__ __forceinline__ bool epi_conv(const TcArgs &a, unsigned char *smem, c
                     pack_e4m3<16>(v, a.mid_inv, r);
                     tmem_st<4>(a2t + c0 / 4, r);
                 }
-            } else if constexpr (C::EPI == EPI_UP) {
-                if constexpr (CAL) amax_fold(a.amax, a.amax_mid, v, valid);
-                unsigned char *a2 = smem + C::OFF_A2 + ab * C::A2_BYTES;
-                put16<C::PREC>(a2 + ((c0 / C::PW) * kTileM + m) * 16, (size_t)kTileM * 16, v, a.mid_inv);
             } else {
                 if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid);
                 unsigned char *dst = a.out + planar_off(e, ((int)blockIdx.x % C::NSPLIT) * C::POUT + c0 / C::PW,
@@ -769,9 +753,9 @@ __device__ bool epilogue(const TcArgs &a, const ParBlock<C::NPAR> &par, unsigned
     const int m = q * 32 + lane;                    // tile row
     const int wg = (warp - 2) >> 2;                 // epilogue warpgroup
     const uint32_t lane_field = (uint32_t)(q * 32) << 16;
-    const uint32_t a2_lane = tmem + lane_field + C::A2_COL0;    // A2T: this warp's lanes of the A2 buffers
+    const uint32_t a2_lane = tmem + lane_field + C::A2_COL0;    // this warp's lanes of the ConvT's operand buffers
     constexpr int64_t ROWS_P = C::ROWS_P;           // pooled tensor
-    constexpr bool ROLES = C::EPI == EPI_UP && C::EWG >= 2;
+    constexpr bool ROLES = C::EPI == EPI_UP;
     const int ntiles = a.n_events * C::TPE;
     const int part = (int)blockIdx.x % C::NSPLIT;   // this CTA's part of a split layer
     for (int i = 0;; ++i) {
@@ -808,8 +792,7 @@ __device__ bool epilogue(const TcArgs &a, const ParBlock<C::NPAR> &par, unsigned
                                                 valid, sx, a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
                                                 (uint32_t)(i >> 1) * C::xchunks(C::COUT / PER), abort))
                     return false;
-                if constexpr (C::A2T) tmem_st_wait();   // A2 in TMEM complete before the MMA reads it
-                else fence_proxy_async_smem();          // A2 writes -> visible to the tensor core
+                tmem_st_wait();                 // the operand is in TMEM before the MMA reads it
                 tc_fence_before();
                 mbar_arrive(&a2full[ab]);
             } else {            // ConvT accumulator -> output; frees the buffer
@@ -830,19 +813,7 @@ __device__ bool epilogue(const TcArgs &a, const ParBlock<C::NPAR> &par, unsigned
             mbar_arrive(&tempty[b]);
             continue;
         }
-        if constexpr (C::EPI == EPI_UP) {   // one warpgroup: conv, then the ConvT
-            if (!epi_conv<C, C::COUT, CAL>(a, smem, par, C::QB, C::QS, dcol, 0, ab, e, p, m, valid, sx,
-                                      a2_lane + ab * C::A2_COLS, inseq, &xready[ab],
-                                      (uint32_t)(i >> 1) * C::xchunks(C::COUT), abort))
-                return false;
-            if constexpr (C::A2T) tmem_st_wait();
-            else fence_proxy_async_smem();
-            tc_fence_before();
-            mbar_arrive(&a2full[ab]);
-            if (!mbar_wait(&t2full[b], ph_b, abort)) return false;
-            tc_fence_after();
-            epi_up<C, C::N2, CAL>(a, par, C::QB2, C::QS2, dcol, 0, e, p, valid, true);
-        } else {                            // this warpgroup's conv columns
+        if constexpr (C::EPI != EPI_UP) {   // this warpgroup's conv columns
             static_assert(!C::PAIRED || C::EPI == EPI_STORE, "paired stores");
             // paired taps (the wide network's split dec3): E[m] + O[m + 1]
             if (!epi_conv<C, C::EPI_COLS, CAL>(a, smem, par, C::QB + part * C::COUT, C::QS + part * C::COUT, dcol, wg * C::EPI_COLS, ab, e, p, m, valid, sx, 0,
@@ -1012,11 +983,9 @@ template <int PREC> struct Net {
     // the fused-ConvT kernels keep the ConvT operand in TMEM (three accumulator buffers
     // leave room for its two buffers): 59 -> 55, 99 -> 96 and 77 -> 75 us (16-bit forms)
     using Enc4Up3 = Cfg<PREC, 64, 0, 128, 500, EPI_UP, 64, is16(PREC) ? 2 : 4,
-                        is16(PREC) ? 2 : 4, 96, 3, false, false, true>;              // 1
-    using Dec3Up2 = Cfg<PREC, 64, 64, 64, 1000, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false,
-                        true>;                                                         // 1 CTA/SM
-    using Dec2Up1 = Cfg<PREC, 32, 32, 32, 2000, EPI_UP, 16, 3, 2, 96, 3, conv_paired(4, PREC), false,
-                        true>;                                                         // 2
+                        is16(PREC) ? 2 : 4, 96, 3>;              // 1
+    using Dec3Up2 = Cfg<PREC, 64, 64, 64, 1000, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC)>;                                                         // 1 CTA/SM
+    using Dec2Up1 = Cfg<PREC, 32, 32, 32, 2000, EPI_UP, 16, 3, 2, 96, 3, conv_paired(4, PREC)>;                                                         // 2
     using Last = Dec1<PREC, 16, 4000>;                                                  // 2
 };
 
@@ -1029,12 +998,12 @@ template <int PREC> struct NetIv {
                          S3 = kIvLen / 8 + kPad;
     static constexpr int L0 = kSlices * S0 - kPad, L1 = kSlices * S1 - kPad, L2 = kSlices * S2 - kPad,
                          L3 = kSlices * S3 - kPad;
-    using Enc2 = Cfg<PREC, 16, 0, 32, L1, EPI_POOL, 0, 4, 1, 56, 2, false, true, false, S1>;
-    using Enc3 = Cfg<PREC, 32, 0, 64, L2, EPI_POOL, 0, 4, 1, 80, 2, false, true, false, S2>;
+    using Enc2 = Cfg<PREC, 16, 0, 32, L1, EPI_POOL, 0, 4, 1, 56, 2, false, true, S1>;
+    using Enc3 = Cfg<PREC, 32, 0, 64, L2, EPI_POOL, 0, 4, 1, 80, 2, false, true, S2>;
     using Enc4Up3 = Cfg<PREC, 64, 0, 128, L3, EPI_UP, 64, is16(PREC) ? 2 : 4, is16(PREC) ? 2 : 4, 96, 3, false,
-                        false, true, S3>;
-    using Dec3Up2 = Cfg<PREC, 64, 64, 64, L2, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false, true, S2>;
-    using Dec2Up1 = Cfg<PREC, 32, 32, 32, L1, EPI_UP, 16, 3, 2, 128, 3, conv_paired(4, PREC), false, true, S1>;
+                        false, S3>;
+    using Dec3Up2 = Cfg<PREC, 64, 64, 64, L2, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false, S2>;
+    using Dec2Up1 = Cfg<PREC, 32, 32, 32, L1, EPI_UP, 16, 3, 2, 128, 3, conv_paired(4, PREC), false, S1>;
     using Last = Dec1<PREC, 16, L0, S0>;
 };
 
@@ -1050,12 +1019,12 @@ template <int PREC> struct Net32 {
     static constexpr int SP = is16(PREC) ? 4 : 2;            // parts of enc4 and dec3
     using Enc2 = Cfg<PREC, 32, 0, 64, 2000, EPI_POOL, 0, 4, 1, 80, 2, false, true>;
     using Enc3 = Cfg<PREC, 64, 0, 128, 1000, EPI_POOL, 0, 3, 2, 128, 2, false, true>;
-    using Enc4 = Cfg<PREC, 128, 0, 256 / SP, 500, EPI_STORE, 0, 3, 1, 128, 2, false, false, false, 0, SP>;
-    using Up3 = Cfg<PREC, 256, 0, 128, 500, EPI_CONVT, 128, 2, 2, 128, 2, false, false, false, 0, 2>;
+    using Enc4 = Cfg<PREC, 128, 0, 256 / SP, 500, EPI_STORE, 0, 3, 1, 128, 2, false, false, 0, SP>;
+    using Up3 = Cfg<PREC, 256, 0, 128, 500, EPI_CONVT, 128, 2, 2, 128, 2, false, false, 0, 2>;
     using Dec3 = Cfg<PREC, 128, 128, 128 / SP, 1000, EPI_STORE, 0, is16(PREC) ? 2 : 3, 1, 128, 2, is16(PREC),
-                     false, false, 0, SP>;
+                     false, 0, SP>;
     using Up2 = Cfg<PREC, 128, 0, 128, 1000, EPI_CONVT, 64, 3, 2, 128, 2>;
-    using Dec2Up1 = Cfg<PREC, 64, 64, 64, 2000, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC), false, true>;
+    using Dec2Up1 = Cfg<PREC, 64, 64, 64, 2000, EPI_UP, 32, 3, 2, 128, 3, conv_paired(3, PREC)>;
     using Last = Dec1<PREC, 32, 4000>;
 };
 

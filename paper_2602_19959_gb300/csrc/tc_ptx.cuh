@@ -83,15 +83,6 @@ __device__ __forceinline__ void sts16(uint32_t a, uint4 v) {
 __device__ __forceinline__ void sts8(uint32_t a, uint2 v) {
     asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
 }
-// 16 floats at a 16-byte aligned shared address that the kernel's prologue filled.
-__device__ __forceinline__ void lds16_at(uint32_t a, float (&v)[16]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        asm("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-            : "=f"(v[4 * i]), "=f"(v[4 * i + 1]), "=f"(v[4 * i + 2]), "=f"(v[4 * i + 3])
-            : "r"(a + 16 * i));
-}
-
 // Longest any wait may take before the kernel gives up (1 s).
 constexpr uint64_t kWaitLimitNs = 1000000000ull;
 
