@@ -11,10 +11,10 @@
 //
 // Each CTA computes a tile of TP positions x all C_out channels of NS sequences (an event
 // is one sequence; the per-interval layout's 40 short sequences go NS = 4 or 8 to a CTA,
-// so that a CTA keeps 128 threads); each thread owns an 8 x 8 register block (8
-// consecutive positions x 8 channels; the ConvT 8 x 16). Inputs are staged through shared
-// memory in chunks of KC channels, transposed to [channel][position] so a thread's 12
-// halo'd inputs are three aligned float4 loads; the weights of the chunk sit next to them
+// so that a CTA keeps 128 threads); each thread owns a PP x 8 register block (PP = 8, or 4 in
+// small launches, consecutive positions x 8 channels; the ConvT 8 x 16). Inputs are staged through shared
+// memory in chunks of KC channels, transposed to [channel][position] so a thread's PP + 4
+// halo'd inputs are aligned float4 loads; the weights of the chunk sit next to them
 // as [tap][channel][C_out]. The sum over (channel, tap) runs in a fixed order: results are
 // deterministic.
 //
@@ -58,13 +58,13 @@ template <int COUT> __device__ __forceinline__ int col_of(int cg, int j) {
     return (j < 4 ? 0 : COUT / 2) + 4 * cg + (j & 3);
 }
 
-template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC>
-__global__ void __launch_bounds__((TP / 8) * (COUT / 8) * NS, 512 / ((TP / 8) * (COUT / 8) * NS))
+template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC, int PP>
+__global__ void __launch_bounds__((TP / PP) * (COUT / 8) * NS, 512 / ((TP / PP) * (COUT / 8) * NS))
 k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
             const float *__restrict__ W, const float *__restrict__ bias,
             float *__restrict__ out, float *__restrict__ outp, int L) {
     constexpr int CIN = CA + CB;
-    constexpr int NCG = COUT / 8, NPG = TP / 8, NT = NCG * NPG * NS;
+    constexpr int NCG = COUT / 8, NPG = TP / PP, NT = NCG * NPG * NS;
     constexpr int XR = TP + 4;              // halo'd rows of a sequence's tile
     constexpr int XP = row_pitch(NS * XR);
     static_assert(CA % KC == 0 && CB % KC == 0 && KC % 4 == 0, "channel chunks must not straddle");
@@ -100,12 +100,12 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
     };
 
     stage_w(0, 0);      // the handle's, like the biases; the inputs are the previous kernel's output
-    float2 acc[8][4];                        // [position][channel pair]
+    float2 acc[PP][4];                        // [position][channel pair]
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const float2 b = make_float2(bias[col_of<COUT>(cg, 2 * q)], bias[col_of<COUT>(cg, 2 * q + 1)]);
 #pragma unroll
-        for (int pi = 0; pi < 8; ++pi) acc[pi][q] = b;
+        for (int pi = 0; pi < PP; ++pi) acc[pi][q] = b;
     }
 
     grid_dep_wait();
@@ -122,10 +122,10 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
         }
 #pragma unroll 4   // against 1: dec3 664 -> 652, dec2 350 -> 339, enc2 107 -> 100 us (500 events)
         for (int k = 0; k < KC; ++k) {
-            float xv[12];
-            const float4 *xr = reinterpret_cast<const float4 *>(&xs[buf][k][sq * XR + pg * 8]);
+            float xv[PP + 4];
+            const float4 *xr = reinterpret_cast<const float4 *>(&xs[buf][k][sq * XR + pg * PP]);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
+            for (int i = 0; i < PP / 4 + 1; ++i) {
                 const float4 v = xr[i];
                 xv[4 * i] = v.x; xv[4 * i + 1] = v.y; xv[4 * i + 2] = v.z; xv[4 * i + 3] = v.w;
             }
@@ -136,7 +136,7 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
                 const float2 wv[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
                                       make_float2(wb.z, wb.w)};
 #pragma unroll
-                for (int pi = 0; pi < 8; ++pi) {
+                for (int pi = 0; pi < PP; ++pi) {
                     const float2 x2 = make_float2(xv[pi + t], xv[pi + t]);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) acc[pi][q] = __ffma2_rn(x2, wv[q], acc[pi][q]);
@@ -148,10 +148,10 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
     const int64_t e = e0 + sq;
     float *ob = out + (size_t)e * rowsE * COUT;
 #pragma unroll
-    for (int pi = 0; pi < 8; ++pi) {
+    for (int pi = 0; pi < PP; ++pi) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[pi][q] = make_float2(leaky(acc[pi][q].x), leaky(acc[pi][q].y));
-        const int p = p0 + pg * 8 + pi;
+        const int p = p0 + pg * PP + pi;
         if (p < L) {
             float *d = ob + (size_t)(p + kPad) * COUT + 4 * cg;
             *reinterpret_cast<float4 *>(d) = make_float4(acc[pi][0].x, acc[pi][0].y, acc[pi][1].x, acc[pi][1].y);
@@ -163,8 +163,8 @@ k_conv5_f32(const float *__restrict__ inA, const float *__restrict__ inB,
         const int Lp = L / 2;
         float *pb = outp + (size_t)e * padded_rows(Lp) * COUT;
 #pragma unroll
-        for (int pi = 0; pi < 8; pi += 2) {
-            const int p = p0 + pg * 8 + pi;
+        for (int pi = 0; pi < PP; pi += 2) {
+            const int p = p0 + pg * PP + pi;
             if (p + 1 < L) {
                 float2 v[4];
 #pragma unroll
@@ -308,12 +308,31 @@ k_convT_f32(const float *__restrict__ in, const float *__restrict__ W,
 // behind the main loop, 234 at the start; 500 events 2333, 2312, 2312, 2366).
 
 // n: sequences (a multiple of NS)
+template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC, int PP>
+cudaError_t conv5_pp(const void *a, const void *b, const float *W, const float *bias, void *out,
+                     void *outp, int L, dim3 grid, cudaStream_t s) {
+    return launch_pdl(k_conv5_f32<CA, CB, COUT, TP, NS, POOL, KC, PP>, grid, dim3((TP / PP) * (COUT / 8) * NS), 0, s,
+                      (const float *)a, (const float *)b, W, bias, (float *)out, (float *)outp, L);
+}
+
 template <int CA, int CB, int COUT, int TP, int NS, bool POOL, int KC>
 cudaError_t conv5(const void *a, const void *b, const float *W, const float *bias, void *out,
                   void *outp, int L, int n, cudaStream_t s) {
-    dim3 grid((L + TP - 1) / TP, n / NS), block((TP / 8) * (COUT / 8) * NS);
-    return launch_pdl(k_conv5_f32<CA, CB, COUT, TP, NS, POOL, KC>, grid, block, 0, s, (const float *)a,
-                      (const float *)b, W, bias, (float *)out, (float *)outp, L);
+    if constexpr (NS == 1) {
+        // tiles of half the positions, half of them per thread, where each has an SM of its own: a
+        // tile is bound by its SM's FMA pipe, which then has half the work (1 event 148 -> 117 us a
+        // call, 9 events 156 -> 125; with up to 1.5 and 2 tiles per SM: 16 events 158 and 157
+        // either way, 8 events of the wide network 271 and 274). Half the positions per thread in
+        // tiles of the same size: no gain
+        int sms = 0;
+        const cudaError_t err = current_device_sms(&sms);
+        if (err != cudaSuccess) return err;
+        const dim3 half((L + TP / 2 - 1) / (TP / 2), n);
+        if ((int64_t)half.x * half.y <= sms)
+            return conv5_pp<CA, CB, COUT, TP / 2, NS, POOL, KC, 4>(a, b, W, bias, out, outp, L, half, s);
+    }
+    const dim3 grid((L + TP - 1) / TP, n / NS);
+    return conv5_pp<CA, CB, COUT, TP, NS, POOL, KC, 8>(a, b, W, bias, out, outp, L, grid, s);
 }
 
 template <int CIN, int COUT, int TP, int NS, int KC>
