@@ -287,7 +287,9 @@ __device__ __forceinline__ void enc_epi(const EncPool &L, const P &par, const Tc
             ldp(par, L.scale + c0, sc);
             scale_bias_leaky(v, sc, bj);
         }
-        if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, valid);
+        // stored rows only: a recomputed tile of a split event has rows whose inputs nobody in this
+        // unit wrote, and every row is stored by one unit
+        if constexpr (CAL) amax_fold(a.amax, a.amax_out, v, st);
         uint4 w = make_uint4(0, 0, 0, 0);
         if constexpr (is16(PREC)) {
             using T = typename Elem<PREC>::T;
