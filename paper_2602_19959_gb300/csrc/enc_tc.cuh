@@ -98,14 +98,6 @@ template <class E>
 __device__ bool enc_producer(const EncArgs &a, unsigned char *smem, uint64_t *bar, volatile int *abort) {
     using C = typename E::C2;
     uint64_t *full = bar + E::FULL, *empty = bar + E::EMPTY;
-    mbar_arrive_expect_tx(bar + E::W2, C::W_BYTES);
-    bulk_g2s(smem + E::OFF_W2, a.c2.w, C::W_BYTES, bar + E::W2);
-    mbar_arrive_expect_tx(bar + E::W3, E::C3::W_BYTES);
-    bulk_g2s(smem + E::OFF_W3, a.c3.w, E::C3::W_BYTES, bar + E::W3);
-    mbar_arrive_expect_tx(bar + E::W4, E::C4::W_BYTES + E::C4::W2_BYTES);
-    bulk_g2s(smem + E::OFF_W4, a.c4.w, E::C4::W_BYTES, bar + E::W4);
-    bulk_g2s(smem + E::OFF_W5, a.c4.w2, E::C4::W2_BYTES, bar + E::W4);
-    grid_dep_wait();      // the weights are the handle's; p1 (and a device-side count) the previous kernel's
     const int n_ev = launch_events(a.c2.n_dyn, a.c2.dyn_base, a.c2.n_events);
     const int lg = enc_split(n_ev, gridDim.x), nu = n_ev << lg;
     int n = 0;
@@ -414,6 +406,14 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
         }
         *abort = 0;
         fence_mbar_init();
+        // the weights are the handle's: they load before the previous kernel has finished
+        mbar_arrive_expect_tx(bar + E::W2, C2::W_BYTES);
+        bulk_g2s(smem + E::OFF_W2, g.c2.w, C2::W_BYTES, bar + E::W2);
+        mbar_arrive_expect_tx(bar + E::W3, C3::W_BYTES);
+        bulk_g2s(smem + E::OFF_W3, g.c3.w, C3::W_BYTES, bar + E::W3);
+        mbar_arrive_expect_tx(bar + E::W4, C4::W_BYTES + C4::W2_BYTES);
+        bulk_g2s(smem + E::OFF_W4, g.c4.w, C4::W_BYTES, bar + E::W4);
+        bulk_g2s(smem + E::OFF_W5, g.c4.w2, C4::W2_BYTES, bar + E::W4);
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, E::TMEM_COLS);
@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(E::THREADS, 1) k_enc_tc(const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (warp != 0 || lane != 0) grid_dep_wait();   // the producer waits after it has asked for the weights
+    grid_dep_wait();      // p1 (and a device-side count) are the previous kernel's output
     grid_dep_launch();
     bool ok = true;
     if (warp == 0) {
