@@ -6,12 +6,11 @@ A launch's schedule has two kinds of free parameters:
     give each layer kernel more tiles per SM and fewer launches;
   * the grids: how many CTAs per SM each persistent kernel family launches (pvf_schedule:
     the front, whose grid sets the events each CTA walks and, in the tensor-core forms,
-    the FC tile (passes of 256 tracks at 1-2 CTAs per SM, 128 at 3-4), the six tensor-core conv
-    kernels, whose grids set the tiles per CTA, and the peak finder; the three encoder entries
-    act in the per-interval layout and the wide network only, where they are kernels of their
-    own). More resident CTAs
+    the FC tile (passes of 256 tracks at 1-2 CTAs per SM, 128 at 3-4), the tensor-core conv
+    kernels, whose grids set the tiles per CTA, and the peak finder). More resident CTAs
     hide latency; fewer leave each CTA more shared-memory and register headroom and
-    shorten the tail of the last wave.
+    shorten the tail of the last wave. Only values that change a launch are tried
+    (grid_candidates): a measured difference between two equal launches is noise.
 For a workload the tuner captures the whole batch as one CUDA graph per candidate, times
 graph launches with CUDA events (L2 flushed between launches), and walks the parameters
 one at a time (coordinate descent), keeping each parameter at its fastest value before
@@ -25,11 +24,26 @@ import json
 import os
 
 FAMILIES = ("front", "enc2", "enc3", "enc4_up3", "dec3_up2", "dec2_up1", "dec1_final", "tail")
-# CTAs per SM tried for each family (0 = as many as fit; the library clamps larger values)
-GRID_CANDIDATES = {"front": (1, 2, 3, 4), "enc2": (2, 3, 4, 6), "enc3": (1, 2, 3, 4), "enc4_up3": (1,),
-                   "dec3_up2": (1,), "dec2_up1": (1, 2), "dec1_final": (2, 3, 4, 5),
-                   "tail": (1, 2, 4)}
+# CTAs per SM tried for each family, by form and UNet base width, beside 0 (as many as fit): those
+# values that are below what fits an SM. Families left out have no kernel of their own (the encoder
+# of whole events at width 16 is one kernel of one CTA per SM; the float32 form has no conv entries)
+# or only one CTA that fits.
+_FRONT = (1, 2, 3, 4)           # 1-2 and 3-4 are two shapes of the kernel
+GRID_CANDIDATES = {
+    ("fp32", 16): {"front": (1,), "tail": (1,)},
+    ("fp32", 32): {"front": (1,), "tail": (1,)},
+    ("16-bit", 16): {"front": _FRONT, "dec2_up1": (1,), "dec1_final": (1,), "tail": (1, 2)},
+    ("16-bit", 32): {"front": _FRONT, "enc2": (2, 3), "tail": (1, 2)},
+    ("fp8", 16): {"front": _FRONT, "dec3_up2": (1,), "dec2_up1": (1, 2), "dec1_final": (1,), "tail": (1, 2)},
+    ("fp8", 32): {"front": _FRONT, "enc2": (2, 3), "enc3": (1,), "enc4_up3": (1,), "dec3_up2": (1,), "dec2_up1": (1,),
+                  "tail": (1, 2)},
+}
 TUNED_DIR = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned")
+
+
+def grid_candidates(precision, width):
+    """{family: CTAs per SM to try} for whole events of this form and UNet base width."""
+    return GRID_CANDIDATES["16-bit" if precision in ("bf16", "fp16") else precision, width]
 
 
 def _time_graph(pv, feats, offs, repeats, warmup, flush):
@@ -57,6 +71,7 @@ def tune(weights, batch, precision="bf16", chunk_candidates=(0,), repeats=3, war
     Returns (best: dict with "chunk_events" and the schedule, trials: list of dicts)."""
     import torch
     from .pvf import PVFinder
+    from .weights import unet_width
 
     n = batch.n_events
     feats = torch.from_numpy(batch.features).cuda()
@@ -88,8 +103,8 @@ def tune(weights, batch, precision="bf16", chunk_candidates=(0,), repeats=3, war
             ms = measure(c, sched)
             if ms < best_ms:
                 best_ms, chunk = ms, c
-        for fam in FAMILIES:
-            for v in GRID_CANDIDATES[fam]:
+        for fam, values in grid_candidates(precision, unet_width(weights)).items():
+            for v in values:
                 cand = dict(sched, **{fam: v})
                 ms = measure(chunk, cand)
                 if ms < best_ms:
