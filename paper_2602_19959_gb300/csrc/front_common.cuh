@@ -1,5 +1,5 @@
 // Device code shared by the front kernels (k_front.cu: CUDA-core FC for the FP32 form and
-// the static-scratch histogram; k_front_tc.cu: tcgen05 FC for the BF16 and FP8 forms):
+// the static-scratch histogram; k_front_tc.cu: tcgen05 FC for the tensor-core forms):
 // event validation, the stable slice sort, and enc1 + pool with its stores.
 #pragma once
 

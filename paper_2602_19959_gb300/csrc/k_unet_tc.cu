@@ -45,10 +45,11 @@
 // resets the counter for the next launch. In the other kernels the ring's handshake per
 // tile measured slower than the imbalance it removes.
 //
-// Launch: programmatic dependent launch. The prologue (weights, parameters, barriers,
-// TMEM) runs before griddepcontrol.wait, i.e. while the previous kernel finishes; the
-// kernel then lets the next one launch. Every wait is bounded (1 s); on timeout the
-// kernel records PVF_ERR_TIMEOUT, drains its own copies and MMAs, frees TMEM and returns.
+// Launch: programmatic dependent launch. The prologue (barriers, TMEM; in k_enc_tc and
+// k_dec1_tc the weight copies too) runs before griddepcontrol.wait, i.e. while the previous
+// kernel finishes; the kernel then lets the next one launch. Every wait is bounded (1 s); on
+// timeout the kernel records PVF_ERR_TIMEOUT, drains its own copies and MMAs, frees TMEM and
+// returns.
 #include "pvf_tc.cuh"
 #include "tc_ptx.cuh"
 
@@ -145,7 +146,6 @@ struct Cfg {
     // the epilogue has read before the ConvT's operand is complete
     static constexpr int CONV_COLS = PAIRED ? 2 * COUT : COUT;      // E | O when paired
     static constexpr int COLS_BUF = CONV_COLS > N2 ? CONV_COLS : N2;
-    static constexpr int UP_OFF = 0;
     static constexpr int A2_COL0 = NB * COLS_BUF;            // A2 buffers after the accumulators
     static constexpr int TMEM_COLS = pow2ceil(NB * COLS_BUF + 2 * A2_COLS);
     // launch parameters: bias (every part's), bias2, and for e4m3 their column scales
@@ -419,11 +419,6 @@ __device__ __forceinline__ void issue_up_ts(uint32_t d2, uint32_t a2_tmem, uint3
     }
 }
 
-template <class C>
-__device__ __forceinline__ void issue_up_any(uint32_t tmem, int bp, int ap, uint32_t w2_base) {
-    issue_up_ts<C>(tmem + bp * C::COLS_BUF + C::UP_OFF, tmem + C::A2_COL0 + ap * C::A2_COLS, w2_base);
-}
-
 // One thread issues all MMAs. With a fused ConvT,
 // the conv of tile i is issued before the ConvT of tile i - 1, so the tensor core works while
 // the epilogue turns tile i - 1's conv accumulator into the operand of its ConvT. The ring
@@ -464,7 +459,7 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
                 const int ap = (i - 1) & 1;
                 if (!mbar_wait(&a2full[ap], ((i - 1) >> 1) & 1, abort)) { ok = false; break; }
                 tc_fence_after();
-                issue_up_any<C>(tmem, bp, ap, w2_base);
+                issue_up_ts<C>(tmem + bp * C::COLS_BUF, tmem + C::A2_COL0 + ap * C::A2_COLS, w2_base);
                 mma_commit(&t2full[bp]);
             }
             bp = b;
@@ -477,7 +472,7 @@ __device__ bool mma_issuer(const TcArgs &a, unsigned char *smem, uint64_t *bar, 
             const int ap = (i - 1) & 1;
             if (mbar_wait(&a2full[ap], ((i - 1) >> 1) & 1, abort)) {
                 tc_fence_after();
-                issue_up_any<C>(tmem, bp, ap, w2_base);
+                issue_up_ts<C>(tmem + bp * C::COLS_BUF, tmem + C::A2_COL0 + ap * C::A2_COLS, w2_base);
                 mma_commit(&t2full[bp]);
             } else {
                 ok = false;
@@ -553,7 +548,7 @@ __device__ __forceinline__ bool paired_cols(uint32_t dcol, int c0, float *sx, in
 
 // Epilogue pieces, one TMEM lane (tile row m, position p) per thread.
 // Conv columns [c_beg, c_beg + NC) of accumulator dcol: bias, LeakyReLU, then either the
-// fused ConvT's shared-memory operand (A2) or the stored output (+ the 2:1 max-pool).
+// fused ConvT's operand in tensor memory (A2) or the stored output (+ the 2:1 max-pool).
 // inseq: the row is a position of a sequence (false: a zero row between sequences of the
 // per-interval layout, stored as zeros). Paired taps: the exchange of each column chunk
 // meets on xready, which completed xuse0 times before this tile (returns false on a
@@ -697,9 +692,9 @@ __device__ __forceinline__ void epi_up(const TcArgs &a, const P &par, int pbias,
     for (int cc = 0; cc < NC; cc += LDW) {
         float vv[LDW];
         if constexpr (LDW == 32) {
-            tmem_ld32(dcol + C::UP_OFF + n_beg + cc, vv);
+            tmem_ld32(dcol + n_beg + cc, vv);
         } else {
-            tmem_ld16(dcol + C::UP_OFF + n_beg + cc, vv);
+            tmem_ld16(dcol + n_beg + cc, vv);
         }
 #pragma unroll
         for (int h = 0; h < LDW / 16; ++h) {
@@ -885,7 +880,7 @@ k_conv_tc(TcArgs a, const __grid_constant__ ParBlock<C::NPAR> par) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    // the prologue above only touched weights and parameters; the activations are the
+    // the prologue above touched nothing that a kernel writes; the activations are the
     // previous kernel's output
     grid_dep_wait();
     grid_dep_launch();

@@ -559,7 +559,6 @@ static cudaError_t run_chunk(pvf_handle *h, const pvf_tracks_soa *tracks, const 
             t.logit_in = buf.logits;
             t.logit_in_base = ev_base;
         }
-        t.d1_scale = h->act_scale[kScaleD1];
         t.final_w = h->fin;
         t.c0 = h->c0;
         t.iv = h->cfg.per_interval;

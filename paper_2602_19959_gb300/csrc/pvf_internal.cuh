@@ -30,8 +30,8 @@ constexpr int kFcHidden = 32;
 constexpr int kFcOut = 100;
 constexpr int kFcInPad = 12;   // layer-1 input padded to a multiple of 4 floats
 constexpr int kC0 = 16;        // UNet base width; levels have 16, 32, 64, 128 channels
-constexpr int kC0Max = 32;     // widest variant (float32 form only): 32, 64, 128, 256
-// Per-interval layout (float32 form): each interval is a sequence of kIvLen bins, its
+constexpr int kC0Max = 32;     // wide network: 32, 64, 128, 256
+// Per-interval layout: each interval is a sequence of kIvLen bins, its
 // kSliceBins bins with kIvPad zero bins on each side (the fewest that survive 3 poolings).
 constexpr int kIvPad = 2;
 constexpr int kIvLen = kSliceBins + 2 * kIvPad;
@@ -79,10 +79,6 @@ __host__ __device__ constexpr int fc_img_off(int l) {
 // enc1 (1 -> 16, k5) in float32: W[t][co] then b[co].
 constexpr int kEnc1Floats = 5 * kC0 + kC0;
 constexpr int kEnc1FloatsMax = 6 * kC0Max;
-// final (16 -> 1, k5) in float32: W[t][ci] then b.
-constexpr int kFinalFloats = 5 * kC0 + 1;
-constexpr int kFinalFloatsMax = 5 * kC0Max + 1;
-
 // Device status word values are pvf_status codes; kernels raise them with atomicMax
 // (an integer maximum: order-independent).
 __device__ __forceinline__ void raise_status(int32_t *word, int32_t s) {
@@ -156,29 +152,6 @@ template <> __device__ __forceinline__ uint32_t max2<__half>(uint32_t a, uint32_
 // 8 floats as one 16-byte row of T.
 template <class T> __device__ __forceinline__ uint4 pack8(const float *v) {
     return make_uint4(pack2<T>(v[0], v[1]), pack2<T>(v[2], v[3]), pack2<T>(v[4], v[5]), pack2<T>(v[6], v[7]));
-}
-
-template <class T> __device__ __forceinline__ T to_elem(float v, float inv_scale);
-template <> __device__ __forceinline__ float to_elem<float>(float v, float) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 to_elem<__nv_bfloat16>(float v, float) {
-    return __float2bfloat16_rn(v);
-}
-template <> __device__ __forceinline__ __half to_elem<__half>(float v, float) {
-    return __ushort_as_half((unsigned short)(pack2<__half>(v, 0.0f) & 0xFFFFu));
-}
-template <> __device__ __forceinline__ __nv_fp8_e4m3 to_elem<__nv_fp8_e4m3>(float v, float inv) {
-    return __nv_fp8_e4m3(v * inv);   // saturating round-to-nearest-even
-}
-template <class T> __device__ __forceinline__ float from_elem(T v, float scale);
-template <> __device__ __forceinline__ float from_elem<float>(float v, float) { return v; }
-template <> __device__ __forceinline__ float from_elem<__nv_bfloat16>(__nv_bfloat16 v, float) {
-    return __bfloat162float(v);
-}
-template <> __device__ __forceinline__ float from_elem<__half>(__half v, float) {
-    return __half2float(v);
-}
-template <> __device__ __forceinline__ float from_elem<__nv_fp8_e4m3>(__nv_fp8_e4m3 v, float s) {
-    return float(v) * s;
 }
 
 // Events one launch processes. Without a device-side count (n_dyn null) that is the
@@ -255,7 +228,7 @@ struct FrontArgs {
     int32_t n_events;            // events in this launch
     int32_t ev_base;             // global index of the launch's first event
     int32_t max_tracks;          // per-event cap
-    int32_t c0;                  // UNet base width (16, or 32 in the float32 form)
+    int32_t c0;                  // UNet base width (16 or 32)
     int32_t iv;                  // per-interval layout: e1 / p1 as kSlices sequences per event
     float edge;                  // boundary-track width in mm (0: every track in one slice)
     float edge_hi;               // 10 - edge, rounded to float
@@ -287,9 +260,8 @@ struct TailArgs {
     const void *d1;              // chunk-local padded [n][4004][c0], or null for logit_in
     const float *logit_in;       // non-null: peaks only, read logits
     int32_t logit_in_base;       // event index of logit_in's first row (0: global rows)
-    float d1_scale;              // fp8 only
     const float *final_w;        // 5 c0 + 1 floats: W[t][ci], then b
-    int32_t c0;                  // width of d1 (16, or 32 in the float32 form)
+    int32_t c0;                  // width of d1 (16 or 32)
     int32_t iv;                  // per-interval layout: d1 holds kSlices sequences per event
     int32_t n_events;
     int32_t ev_base;
@@ -359,7 +331,7 @@ __host__ __device__ __forceinline__ int front_entries(int max_tracks, float edge
     return edge > 0.0f ? 2 * max_tracks : max_tracks;
 }
 size_t front_smem_bytes(int max_tracks, float edge);
-// Steps 1-2 + enc1 with the FC on tcgen05 (BF16 and FP8 forms).
+// Steps 1-2 + enc1 with the FC on tcgen05 (the tensor-core forms).
 cudaError_t launch_front_tc(const FrontArgs &a, int precision, cudaStream_t s);
 // Steps 1-2 only (validate, sort, FC, histogram into a.hist_out), float32; e1/p1 unused.
 cudaError_t launch_front_hist_only(const FrontArgs &a, size_t smem_bytes, cudaStream_t s);

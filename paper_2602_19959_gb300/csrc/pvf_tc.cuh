@@ -20,7 +20,7 @@ enum {
     kScaleL1 = 0,   // e1, p1, u1 (level 1, 16 channels)
     kScaleL2 = 1,   // e2, p2, u2
     kScaleL3 = 2,   // e3, p3, u3
-    kScaleE4 = 3,   // e4 (shared-memory operand of the fused up3 GEMM)
+    kScaleE4 = 3,   // e4 (operand of the fused up3 GEMM)
     kScaleD3 = 4,   // d3 (operand of the fused up2 GEMM)
     kScaleD2 = 5,   // d2 (operand of the fused up1 GEMM)
     kScaleD1 = 6,   // d1 (input of the final conv)
