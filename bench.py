@@ -177,7 +177,7 @@ def roofline_of(name, launches, tot_ms, form, events_per_launch, tracks_per_laun
 # commands). Keyed by (form, kernel, events per launch); the value is (bytes, source). A
 # kernel changed since its capture has no entry and reports null.
 NCU_TRAFFIC = {
-    ("fp16", "enc_up3", 1000): ((65.172224e6 + 321.375232e6),
+    ("fp16", "enc_up3", 1000): ((65.246208e6 + 323.6864e6),
                                 "ncu of one 1000-event launch (profiles/kernels_fp16_1000ev.md)"),
     ("fp16", "dec3_up2", 1000): ((257.167104e6 + 87.38432e6),
                                  "ncu of one 1000-event launch (profiles/kernels_fp16_1000ev.md)"),
